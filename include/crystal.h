@@ -88,8 +88,8 @@ int crys_debug_stall(int op, int32_t first_tile, int64_t wait_limit_ns);
  *   order_preserving
  *              0: the paper's scheme, one atomic reservation per tile — tiles land in
  *                 completion order, values inside a tile keep input order.  No scratch.
- *              1: tiles are chained by a decoupled look-back scan so that `out` is in
- *                 input order.  Needs scratch (see conventions).
+ *              1: one block of the launch turns the tiles' counts into positions in tile
+ *                 order, so that `out` is in input order.  Needs scratch (see conventions).
  */
 int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, int32_t* out,
                 int64_t* d_count, int order_preserving, void* d_temp, size_t* temp_bytes,
