@@ -200,17 +200,18 @@ int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out,
               int32_t* vals_out, int64_t n, void* d_temp, size_t* temp_bytes, crys_stream s);
 
 /* Most-significant-digit radix sort (Section 4.4: the GPU sort behind the paper's sort
- * figure is an MSB radix sort, not stable).  Two 8-bit partition passes on the top two
- * digits (signed order: the sign bit is flipped), each a histogram, a scan and a scatter
- * whose tiles rank their keys with shared-memory atomics and reserve each digit's run with
- * one global atomic; then every bucket of the top 16 bits is sorted inside one thread
- * block by the low 16 bits (4 stable passes of 4 bits in shared memory) and stored.
+ * figure is an MSB radix sort, not stable).  None, one or two partition passes of at most 8
+ * bits (n <= 4992, n <= 2^20, larger), each a histogram, a scan and a scatter whose tiles
+ * rank their keys with shared-memory atomics and reserve each digit's run with one global
+ * atomic; then every bucket is sorted inside one thread block by its remaining bits and
+ * stored.  The passes' bits are those of a key's place between the smallest and the largest
+ * key of a sample, so narrow key ranges fill the buckets like wide ones.
  * Keys come out in ascending signed order; rows with EQUAL keys may come out in any order
  * (unstable), so (key, value) pairs are a permutation of the input pairs.  A bucket of
- * more than 8192 rows (heavily repeated top bits) is sorted by one block through global
- * memory: correct for every input, slow only for such skew.  n <= 2^31 - 1; keys_out /
+ * more than 4992 rows (heavily repeated or clustered keys) is sorted by one block through
+ * global memory: correct for every input, slow only for such skew.  n <= 2^31 - 1; keys_out /
  * vals_out must not overlap the inputs.  Scratch (two-call size query): n keys + n values
- * plus about 1.3 MB of bucket arrays. */
+ * plus at most 1.1 MB of bucket arrays. */
 int crys_sort_msb(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out,
                   int32_t* vals_out, int64_t n, void* d_temp, size_t* temp_bytes, crys_stream s);
 

@@ -1,73 +1,93 @@
 // Radix partitioning without stability, and the two operators built on it:
 //
 //  * crys_sort_msb - the most-significant-digit radix sort the paper's GPU sort number
-//    comes from (Section 4.4): two 8-bit partition passes on the top digits, then every
-//    bucket of the top 16 bits is sorted inside one thread block (shared memory) by the
-//    low 16 bits.  Unstable, as in the paper.
+//    comes from (Section 4.4): one or two partition passes on the leading bits, then every
+//    bucket is sorted inside one thread block (localsort.cuh).  Unstable, as in the paper.
 //  * crys_join_partitioned - the radix-partitioned hash join Section 4.3 sets beside the
 //    no-partitioning join for build sides far beyond the caches: both sides are split by
 //    hash bits in two passes so that each build partition's table fits in shared memory,
 //    then each partition is built and probed there.
 //
-// A partition pass moves (key, value) pairs by an 8-bit digit of the key inside each of
-// up to 65536 segments (the buckets of the previous pass): a histogram kernel counts the
-// digits of every tile, a scan kernel turns the counts into the start of every (segment,
-// digit) bucket, and a scatter kernel ranks a tile's pairs by digit with per-warp
-// shared-memory counters (atomic, hence unstable), reserves each digit's run of the tile
-// with one global atomic per digit, sorts the tile in shared memory and stores each run
-// with consecutive addresses.  No pass waits on another block, so nothing here spins.
+// A partition pass moves (key, value) pairs by a digit of at most 8 bits inside each of up
+// to 256 segments (the buckets of the previous pass): a histogram kernel counts the digits
+// of every segment, a scan kernel turns the counts into the start of every (segment, digit)
+// bucket, and a scatter kernel ranks a tile's pairs by digit with shared-memory atomics
+// (hence unstable), reserves each digit's run of the tile with one global atomic per digit,
+// sorts the tile in shared memory and stores each run with consecutive addresses.  No pass
+// waits on another block, so nothing here spins.
 #include "common.cuh"
+#include "keyrange.cuh"
+#include "localsort.cuh"
 
 namespace crys {
 namespace {
 
 constexpr int kBuckets = 256;
-constexpr int kPartThreads = 256;
-constexpr int kPartItems = 8;
+constexpr int kHistThreads = 256;
+constexpr int kHistItems = 8;
+constexpr int kPartThreads = 512;
+constexpr int kPartItems = 12;
 constexpr int kPartTile = kPartThreads * kPartItems;  // rows per tile of a partition pass
 
-// Digit of a key: ((key * mult) >> shift) & mask, then XOR flip.  Sort digits use
-// mult = 1 (flip 0x80 on the top digit for signed order); join digits use the bits of
-// the multiplicative hash key * 2654435769 from the top down.
-struct DigitFn {
-  uint32_t mult, shift, mask, flip;
-  __host__ __device__ __forceinline__ uint32_t operator()(int32_t k) const {
-    return (((static_cast<uint32_t>(k) * mult) >> shift) & mask) ^ flip;
+// Join digits: bits of the multiplicative hash key * 2654435769 from the top down.
+struct HashDigit {
+  uint32_t shift, mask;
+  __device__ __forceinline__ HashDigit load() const { return *this; }
+  __device__ __forceinline__ uint32_t operator()(int32_t k) const {
+    return ((static_cast<uint32_t>(k) * 2654435769u) >> shift) & mask;
   }
 };
 
+// Sort digits: bits of the key's place in the key range (keyrange.cuh).
+struct RangeDigit {
+  const KeyRange* range;
+  uint32_t shift, mask;
+  struct Fn {
+    KeyRange r;
+    uint32_t shift, mask;
+    __device__ __forceinline__ uint32_t operator()(int32_t k) const { return (r.place(k) >> shift) & mask; }
+  };
+  __device__ __forceinline__ Fn load() const { return Fn{*range, shift, mask}; }
+};
+
 // Segments of a pass: segment s covers rows [begin[s], begin[s] + size[s]) and owns the
-// tiles [tile_start[s], tile_start[s + 1]) of the pass (tile_start has count + 1 entries);
-// tile_seg[b] is the segment of tile b (unused when there is one segment).
+// tiles [tile_start[s], tile_start[s + 1]) of the pass (tile_start has count + 1 entries).
 struct Segs {
-  const int64_t* begin;
-  const int64_t* size;
+  const uint32_t* begin;
+  const uint32_t* size;
   const uint32_t* tile_start;
-  const uint32_t* tile_seg;
   int32_t count;
 };
 
-// The segment and rows of tile `b` of a pass: seg = -1 past the last tile.
+// Rows of tile `b`, which belongs to segment `seg`.
 struct TileAt {
-  int seg;
   int valid;
-  int64_t row0;
+  uint32_t row0;
 };
 
-__device__ __forceinline__ TileAt find_tile(const Segs& S, uint32_t b, int tile_rows) {
-  TileAt r{-1, 0, 0};
-  if (b >= S.tile_start[S.count]) return r;
-  const int lo = S.count == 1 ? 0 : static_cast<int>(S.tile_seg[b]);
-  const int64_t t = static_cast<int64_t>(b - S.tile_start[lo]);
-  const int64_t rem = S.size[lo] - t * tile_rows;
-  r.seg = lo;
-  r.row0 = S.begin[lo] + t * tile_rows;
-  r.valid = static_cast<int>(rem < tile_rows ? rem : tile_rows);
-  return r;
+__device__ __forceinline__ TileAt tile_rows(const Segs& S, int seg, uint32_t b, int rows) {
+  const uint32_t off = (b - S.tile_start[seg]) * static_cast<uint32_t>(rows);
+  const uint32_t rem = S.size[seg] - off;
+  return TileAt{static_cast<int>(rem < static_cast<uint32_t>(rows) ? rem : static_cast<uint32_t>(rows)),
+                S.begin[seg] + off};
+}
+
+// Segment of tile `b` (a tile that exists): the last one that starts at or before it and is
+// not empty, by binary search.
+__device__ __forceinline__ int find_segment(const Segs& S, uint32_t b) {
+  int lo = 0, hi = S.count;  // tile_start[lo] <= b < tile_start[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) / 2;
+    if (S.tile_start[mid] <= b)
+      lo = mid;
+    else
+      hi = mid;
+  }
+  return lo;
 }
 
 // Block-wide exclusive scan of one value per thread (THREADS <= 1024); also returns the
-// total.  `tmp` holds one word per warp.
+// total.  `tmp` holds one word per warp and one more.
 template <int THREADS>
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t* tmp, uint32_t* total) {
   constexpr int WARPS = THREADS / kWarp;
@@ -91,42 +111,32 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t x, uint32_t* t
 // ---------------------------------------------------------------- segment set-up
 
 // One segment covering rows [0, n).
-__global__ void seg_init_kernel(int64_t n, int tile_rows, int64_t* begin, int64_t* size, uint32_t* tile_start) {
+__global__ void seg_init_kernel(uint32_t n, int rows, uint32_t* begin, uint32_t* size, uint32_t* tile_start) {
   begin[0] = 0;
   size[0] = n;
   tile_start[0] = 0;
-  tile_start[1] = static_cast<uint32_t>((n + tile_rows - 1) / tile_rows);
+  tile_start[1] = (n + static_cast<uint32_t>(rows) - 1) / static_cast<uint32_t>(rows);
 }
 
-// The buckets of a pass as the segments of the next one: begin/size from the bucket
-// starts and counts, their tile prefix and the segment of every tile (one block of 1024
-// threads, any count).
-__global__ void __launch_bounds__(1024) seg_from_buckets_kernel(const int64_t* bucket_begin, const uint32_t* bucket_count,
-                                                                int n, int tile_rows, int64_t* begin, int64_t* size,
-                                                                uint32_t* tile_start, uint32_t* tile_seg) {
+// Tile prefix of `n` segments from their sizes (one block of 1024 threads, any n: each
+// thread sums a contiguous share, one block scan joins the shares).
+__global__ void __launch_bounds__(1024) tile_prefix_kernel(const uint32_t* size, int n, int rows, uint32_t* tile_start) {
   __shared__ uint32_t tmp[kWarp + 1];
-  __shared__ uint32_t carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int base = 0; base < n; base += 1024) {
-    const int i = base + static_cast<int>(threadIdx.x);
-    uint32_t tiles = 0;
-    if (i < n) {
-      begin[i] = bucket_begin[i];
-      size[i] = bucket_count[i];
-      tiles = (bucket_count[i] + static_cast<uint32_t>(tile_rows) - 1) / static_cast<uint32_t>(tile_rows);
+  const int share = (n + 1023) / 1024;
+  const int i0 = static_cast<int>(threadIdx.x) * share;
+  auto tiles = [&](int i) {
+    return i < n ? (size[i] + static_cast<uint32_t>(rows) - 1) / static_cast<uint32_t>(rows) : 0u;
+  };
+  uint32_t sum = 0;
+  for (int j = 0; j < share; ++j) sum += tiles(i0 + j);
+  uint32_t total;
+  uint32_t run = block_exclusive_scan<1024>(sum, tmp, &total);
+  for (int j = 0; j < share; ++j)
+    if (i0 + j < n) {
+      tile_start[i0 + j] = run;
+      run += tiles(i0 + j);
     }
-    uint32_t total;
-    const uint32_t ex = block_exclusive_scan<1024>(tiles, tmp, &total);
-    if (i < n) tile_start[i] = carry + ex;
-    __syncthreads();
-    if (threadIdx.x == 0) carry += total;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) tile_start[n] = carry;
-  __syncthreads();
-  for (int i = threadIdx.x; i < n; i += 1024)
-    for (uint32_t t = tile_start[i]; t < tile_start[i + 1]; ++t) tile_seg[t] = static_cast<uint32_t>(i);
+  if (threadIdx.x == 0) tile_start[n] = total;
 }
 
 // ---------------------------------------------------------------- one partition pass
@@ -134,368 +144,180 @@ __global__ void __launch_bounds__(1024) seg_from_buckets_kernel(const int64_t* b
 // Digit counts of every segment.  A persistent block takes a contiguous range of the
 // pass's tiles (so it stays in one segment for many tiles), counts in shared memory and
 // adds its counts to the segment's when the segment changes and at the end.
-__global__ void __launch_bounds__(kPartThreads) part_hist_kernel(const int32_t* __restrict__ keys, Segs S, DigitFn f,
+template <typename Digit>
+__global__ void __launch_bounds__(kHistThreads) part_hist_kernel(const int32_t* __restrict__ keys, Segs S,
+                                                                 const __grid_constant__ Digit digit, int digits,
                                                                  uint32_t* hist) {
   constexpr int kCopies = 4;
+  constexpr int kStep = kHistThreads * kHistItems;
   __shared__ uint32_t h[kCopies][kBuckets];
   const int tid = threadIdx.x;
-  for (int i = tid; i < kCopies * kBuckets; i += kPartThreads) (&h[0][0])[i] = 0;
+  const auto f = digit.load();
+  for (int i = tid; i < kCopies * kBuckets; i += kHistThreads) (&h[0][0])[i] = 0;
   const uint32_t total = S.tile_start[S.count];
   const uint32_t t0 = static_cast<uint32_t>((static_cast<uint64_t>(total) * blockIdx.x) / gridDim.x);
   const uint32_t t1 = static_cast<uint32_t>((static_cast<uint64_t>(total) * (blockIdx.x + 1)) / gridDim.x);
+  if (t0 >= t1) return;
   uint32_t* mine = h[(tid / kWarp) % kCopies];
-  int cur = -1;
-  auto flush = [&](int seg) {
+  const uint64_t pol = policy_evict_first();
+  int seg = find_segment(S, t0);
+  auto flush = [&]() {
     __syncthreads();
-    for (int d = tid; d < kBuckets; d += kPartThreads) {
+    for (int d = tid; d < digits; d += kHistThreads) {
       uint32_t c = 0;
 #pragma unroll
       for (int r = 0; r < kCopies; ++r) {
         c += h[r][d];
         h[r][d] = 0;
       }
-      if (c) atomicAdd(&hist[static_cast<int64_t>(seg) * kBuckets + d], c);
+      if (c) atomicAdd(&hist[seg * digits + d], c);
     }
     __syncthreads();
   };
   __syncthreads();
   for (uint32_t b = t0; b < t1; ++b) {
-    const TileAt at = find_tile(S, b, kPartTile);  // every thread: the same few cached words
-    if (at.seg != cur) {
-      if (cur >= 0) flush(cur);
-      cur = at.seg;
+    if (b >= S.tile_start[seg + 1]) {
+      flush();
+      while (b >= S.tile_start[seg + 1]) ++seg;
     }
-    int32_t k[kPartItems];
+    const TileAt at = tile_rows(S, seg, b, kPartTile);
+    for (int base = 0; base < at.valid; base += kStep) {
+      int32_t k[kHistItems];
 #pragma unroll
-    for (int i = 0; i < kPartItems; ++i) {
-      const int idx = i * kPartThreads + tid;
-      k[i] = idx < at.valid ? keys[at.row0 + idx] : 0;
+      for (int i = 0; i < kHistItems; ++i) {
+        const int idx = base + i * kHistThreads + tid;
+        k[i] = idx < at.valid ? ld_stream(keys + at.row0 + idx, pol) : 0;
+      }
+#pragma unroll
+      for (int i = 0; i < kHistItems; ++i)
+        if (base + i * kHistThreads + tid < at.valid) atomicAdd(&mine[f(k[i])], 1u);
     }
-#pragma unroll
-    for (int i = 0; i < kPartItems; ++i)
-      if (i * kPartThreads + tid < at.valid) atomicAdd(&mine[f(k[i])], 1u);
   }
-  if (cur >= 0) flush(cur);
+  flush();
 }
+
+// A cursor per bucket.  Every tile adds to every cursor of its segment, and adds to one 32-byte
+// sector wait for each other, so the cursors of a first pass, where all tiles share one
+// segment, have a sector each; those of a second pass are four to a sector.
+constexpr int kCursorStrideA = 8, kCursorStrideB = 2;
 
 // Bucket starts of every segment: begin of the segment plus the exclusive prefix of its
 // digit counts.  One block of 256 threads per segment.
-__global__ void __launch_bounds__(kBuckets) part_scan_kernel(const uint32_t* hist, const int64_t* seg_begin,
-                                                             unsigned long long* cursor, int64_t* bucket_begin) {
+__global__ void __launch_bounds__(kBuckets) part_scan_kernel(const uint32_t* hist, const uint32_t* seg_begin, int digits,
+                                                             uint32_t* cursor, int stride, uint32_t* bucket_begin) {
   __shared__ uint32_t tmp[kWarp + 1];
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * kBuckets + threadIdx.x;
+  const int d = threadIdx.x;
+  const int i = static_cast<int>(blockIdx.x) * digits + d;
   uint32_t total;
-  const uint32_t ex = block_exclusive_scan<kBuckets>(hist[i], tmp, &total);
-  const int64_t b = seg_begin[blockIdx.x] + ex;
-  cursor[i] = static_cast<unsigned long long>(b);
-  bucket_begin[i] = b;
+  const uint32_t ex = block_exclusive_scan<kBuckets>(d < digits ? hist[i] : 0u, tmp, &total);
+  if (d < digits) {
+    const uint32_t b = seg_begin[blockIdx.x] + ex;
+    cursor[i * stride] = b;
+    bucket_begin[i] = b;
+  }
 }
 
-constexpr long long kSkipRun = -(1ll << 62);  // a digit run that is reported and dropped
-static_assert(kPartThreads == kBuckets, "one thread per digit in the scatter's bookkeeping");
-
+template <typename Digit>
 struct ScatterArgs {
   const int32_t* kin;
   const int32_t* vin;
   int32_t* kout;
   int32_t* vout;
   Segs S;
-  DigitFn f;
-  unsigned long long* cursor;  // [segments][256] next free row of each bucket
+  Digit digit;
+  int32_t digits;
+  uint32_t* cursor;  // [segments][digits], `stride` words apart: next free row of each bucket
+  int32_t stride;
   int32_t* err;
 };
 
-__global__ void __launch_bounds__(kPartThreads) part_scatter_kernel(const __grid_constant__ ScatterArgs a) {
-  constexpr int WARPS = kPartThreads / kWarp;
+// One tile of 6144 pairs per block, three blocks per SM.  The tile is what a digit's run is
+// cut from (24 rows on average at 256 digits; 2048-row tiles wrote 8-row runs), and the keys
+// and values go through the same registers one after the other, so that three blocks fit
+// and one's loads and barriers hide behind the others' work: at 2^28 pairs 1.01 ms per pass
+// against 1.09 with 8192-row tiles, two blocks per SM and both columns in registers, and
+// 1.50 with 2048-row tiles and counters per warp.  Latency bounds it: issue is active half
+// of the cycles, the L1 pipe 65%, DRAM 40%.
+template <typename Digit>
+__global__ void __launch_bounds__(kPartThreads, 3) part_scatter_kernel(const __grid_constant__ ScatterArgs<Digit> a) {
   extern __shared__ __align__(16) int32_t part_smem[];
   int32_t* sk = part_smem;               // the tile's keys in bucket order
   int32_t* sv = part_smem + kPartTile;   // and values
-  __shared__ uint32_t wh[WARPS][kBuckets];  // per-warp digit counts, then the warps' offsets
-  __shared__ uint32_t lstart[kBuckets];     // tile-local start of each digit's run
-  __shared__ long long gshift[kBuckets];    // global row minus tile-local position, or kSkipRun
+  __shared__ uint32_t count[kBuckets];   // rows of each digit
+  __shared__ uint32_t lstart[kBuckets];  // tile-local start of each digit's run
+  __shared__ uint32_t gshift[kBuckets];  // global row minus tile-local position (mod 2^32)
   __shared__ uint32_t tmp[kWarp + 1];
   __shared__ int seg_sh;
-  __shared__ long long row0_sh, seg_lo_sh, seg_hi_sh;
-  __shared__ int valid_sh;
-  const int tid = threadIdx.x, warp = tid / kWarp;
-  for (int i = tid; i < WARPS * kBuckets; i += kPartThreads) (&wh[0][0])[i] = 0;
-  if (tid == 0) {
-    const TileAt at = find_tile(a.S, blockIdx.x, kPartTile);
-    seg_sh = at.seg;
-    row0_sh = at.row0;
-    valid_sh = at.valid;
-    if (at.seg >= 0) {
-      seg_lo_sh = a.S.begin[at.seg];
-      seg_hi_sh = a.S.begin[at.seg] + a.S.size[at.seg];
-    }
-  }
+  const int tid = threadIdx.x;
+  const uint32_t b = blockIdx.x;
+  if (b >= a.S.tile_start[a.S.count]) return;
+  if (tid < kBuckets) count[tid] = 0;
+  if (tid < a.S.count && a.S.tile_start[tid] <= b && b < a.S.tile_start[tid + 1]) seg_sh = tid;  // one of at most 256
+  const auto f = a.digit.load();
   __syncthreads();
   const int seg = seg_sh;
-  if (seg < 0) return;
-  const int64_t row0 = row0_sh;
-  const int valid = valid_sh;
-  int32_t k[kPartItems], v[kPartItems];
-  uint32_t r[kPartItems];
+  const TileAt at = tile_rows(a.S, seg, b, kPartTile);
+  const uint64_t pol = policy_evict_first();
+  int32_t k[kPartItems];   // keys, then values
+  uint32_t r[kPartItems];  // digit << 16 | rank inside the tile's rows of that digit, then place in the tile
 #pragma unroll
   for (int i = 0; i < kPartItems; ++i) {
     const int idx = i * kPartThreads + tid;
-    k[i] = idx < valid ? a.kin[row0 + idx] : 0;
-    v[i] = idx < valid ? a.vin[row0 + idx] : 0;
+    k[i] = idx < at.valid ? ld_stream(a.kin + at.row0 + idx, pol) : 0;
   }
-  // rank inside the warp's counters (shared-memory atomics: unstable)
+  if (tid == 0) {  // the values are read after the keys are placed: on their way to L2 meanwhile
+    const uint32_t mis = static_cast<uint32_t>((reinterpret_cast<uintptr_t>(a.vin + at.row0) & 15u) / 4);
+    const uint32_t lead = mis ? 4 - mis : 0;
+    const uint32_t words = static_cast<uint32_t>(at.valid) > lead ? (at.valid - lead) & ~3u : 0u;
+    if (words) bulk_prefetch_l2(a.vin + at.row0 + lead, words * 4);
+  }
 #pragma unroll
   for (int i = 0; i < kPartItems; ++i)
-    r[i] = (i * kPartThreads + tid < valid) ? atomicAdd(&wh[warp][a.f(k[i])], 1u) : 0u;
-  __syncthreads();
-  {
-    const int d = tid;  // kPartThreads == kBuckets: one thread per digit
-    uint32_t run = 0;
-#pragma unroll
-    for (int w = 0; w < WARPS; ++w) {
-      const uint32_t c = wh[w][d];
-      wh[w][d] = run;
-      run += c;
+    if (i * kPartThreads + tid < at.valid) {
+      const uint32_t d = f(k[i]);
+      r[i] = (d << 16) | atomicAdd(&count[d], 1u);
     }
+  __syncthreads();
+  bool bad = false;
+  {
+    const uint32_t run = tid < a.digits ? count[tid] : 0u;
     uint32_t total;
     const uint32_t ls = block_exclusive_scan<kPartThreads>(run, tmp, &total);
-    lstart[d] = ls;
-    long long shift = 0;
     if (run) {
-      const long long g = static_cast<long long>(atomicAdd(&a.cursor[static_cast<int64_t>(seg) * kBuckets + d],
-                                                           static_cast<unsigned long long>(run)));
-      // the run must stay inside its segment (it does whenever the counts came from
-      // these keys); otherwise report and drop it rather than write out of place
-      if (g < seg_lo_sh || g + run > seg_hi_sh) {
-        set_error(a.err, CRYS_DEV_BOUNDS);
-        shift = kSkipRun;
-      } else {
-        shift = g - ls;
-      }
+      const uint32_t g = atomicAdd(&a.cursor[(seg * a.digits + tid) * a.stride], run);
+      // the run must stay inside its segment (it does whenever the counts came from these
+      // keys); otherwise the tile is reported and dropped rather than written out of place
+      bad = g < a.S.begin[seg] || g + run > a.S.begin[seg] + a.S.size[seg];
+      if (bad) set_error(a.err, CRYS_DEV_BOUNDS);
+      lstart[tid] = ls;
+      gshift[tid] = g - ls;
     }
-    gshift[d] = shift;
   }
-  __syncthreads();
+  if (__syncthreads_or(bad)) return;
+#pragma unroll
+  for (int i = 0; i < kPartItems; ++i)
+    if (i * kPartThreads + tid < at.valid) {
+      const uint32_t p = lstart[r[i] >> 16] + (r[i] & 0xFFFFu);
+      sk[p] = k[i];
+      r[i] = p;
+    }
 #pragma unroll
   for (int i = 0; i < kPartItems; ++i) {
-    if (i * kPartThreads + tid < valid) {
-      const uint32_t d = a.f(k[i]);
-      const uint32_t p = lstart[d] + wh[warp][d] + r[i];
-      sk[p] = k[i];
-      sv[p] = v[i];
-    }
+    const int idx = i * kPartThreads + tid;
+    k[i] = idx < at.valid ? ld_stream(a.vin + at.row0 + idx, pol) : 0;
   }
+#pragma unroll
+  for (int i = 0; i < kPartItems; ++i)
+    if (i * kPartThreads + tid < at.valid) sv[r[i]] = k[i];
   __syncthreads();
-  for (int j = tid; j < valid; j += kPartThreads) {
+#pragma unroll 4
+  for (int j = tid; j < at.valid; j += kPartThreads) {
     const int32_t key = sk[j];
-    const long long s = gshift[a.f(key)];
-    if (s == kSkipRun) continue;
-    a.kout[s + j] = key;
-    a.vout[s + j] = sv[j];
+    const uint32_t g = gshift[f(key)] + static_cast<uint32_t>(j);
+    a.kout[g] = key;
+    a.vout[g] = sv[j];
   }
 }
-
-// ---------------------------------------------------------------- local sort (MSB sort)
-//
-// Every bucket of the top 16 key bits is sorted by the low 16 bits inside one block.  A
-// bucket of at most kLocalCap rows is sorted in shared memory as (low 16 bits, row)
-// words, 4 stable passes of 4 bits: each thread owns kLocalIpt consecutive words, counts
-// their digits in packed 8-bit counters, a block scan over (digit, thread) gives every
-// thread the first position of each digit, and the thread walks its words in order
-// (stable).  The sorted rows are then gathered from the bucket in global memory (it was
-// just read, so L2 serves the gather) and stored with consecutive addresses.
-
-constexpr int kLocalThreads = 256;
-constexpr int kLocalIpt = 20;
-constexpr int kLocalCap = kLocalThreads * kLocalIpt;  // 5120 rows: a 13-bit row index
-static_assert(kLocalCap <= 8192 && kLocalIpt <= 255, "13-bit rows, 8-bit per-thread digit counters");
-constexpr int kLocalPad = kLocalIpt + 1;              // words per thread slice incl. one pad word
-
-// Position p of the sorted order in the padded layout (one pad word per 16 words, so that
-// the threads' slices start in distinct banks).
-__device__ __forceinline__ int padded(int p) { return p + p / kLocalIpt; }
-
-// One stable 4-bit pass of the words in `src` (cnt valid ones, padded layout) into
-// `dst` by the digit (w >> shift) & 15.  `scan` holds 16 x kLocalThreads counters.
-__device__ __forceinline__ void local_pass(const uint32_t* src, uint32_t* dst, int cnt, int shift, uint32_t* scan,
-                                           uint32_t* tmp) {
-  const int t = threadIdx.x;
-  uint32_t w[kLocalIpt];
-  uint32_t c4[4] = {0u, 0u, 0u, 0u};  // 16 digit counters of 8 bits, packed four to a word
-#pragma unroll
-  for (int i = 0; i < kLocalIpt; ++i) {
-    const int p = t * kLocalIpt + i;
-    w[i] = p < cnt ? src[t * kLocalPad + i] : 0u;
-    if (p < cnt) {
-      const uint32_t d = (w[i] >> shift) & 15u;
-      const uint32_t inc = 1u << (8 * (d & 3u));
-      c4[0] += (d >> 2) == 0 ? inc : 0u;
-      c4[1] += (d >> 2) == 1 ? inc : 0u;
-      c4[2] += (d >> 2) == 2 ? inc : 0u;
-      c4[3] += (d >> 2) == 3 ? inc : 0u;
-    }
-  }
-#pragma unroll
-  for (int d = 0; d < 16; ++d) scan[d * kLocalThreads + t] = (c4[d >> 2] >> (8 * (d & 3))) & 0xFFu;
-  __syncthreads();
-  // exclusive scan of the 16 x kLocalThreads counters in (digit, thread) order: each
-  // thread takes 16 consecutive counters, then one block scan of the threads' sums
-  static_assert(16 * kLocalThreads % kLocalThreads == 0, "16 counters per thread");
-  uint32_t loc[16];
-  uint32_t sum = 0;
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    loc[j] = scan[t * 16 + j];
-    sum += loc[j];
-  }
-  uint32_t total;
-  uint32_t run = block_exclusive_scan<kLocalThreads>(sum, tmp, &total);
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const uint32_t c = loc[j];
-    scan[t * 16 + j] = run;
-    run += c;
-  }
-  __syncthreads();
-  // stable placement: this thread's words in order, each at its digit's next position
-#pragma unroll
-  for (int i = 0; i < kLocalIpt; ++i) {
-    if (t * kLocalIpt + i < cnt) {
-      const uint32_t d = (w[i] >> shift) & 15u;
-      uint32_t* slot = &scan[d * kLocalThreads + t];
-      const uint32_t p = *slot;
-      *slot = p + 1;
-      dst[padded(static_cast<int>(p))] = w[i];
-    }
-  }
-  __syncthreads();
-}
-
-struct LocalArgs {
-  const int32_t* kin;  // buckets of the top 16 bits (after two partition passes)
-  const int32_t* vin;
-  int32_t* kout;
-  int32_t* vout;
-  const int64_t* bucket_begin;   // [65536]
-  const uint32_t* bucket_count;  // [65536]
-  int32_t* err;
-};
-
-// Rows of a bucket larger than kLocalCap: sorted by one block through global memory,
-// 4 stable passes of 4 bits over chunks of kLocalCap rows (the digit starts of the whole
-// bucket carried from chunk to chunk), kin -> kout -> kin -> kout -> kin, then copied
-// to kout.  Correct for every input; a bucket this large means heavily repeated top bits.
-__device__ void local_sort_large(const LocalArgs& a, int64_t begin, int64_t size, uint32_t* words, uint32_t* scan,
-                                 uint32_t* tmp) {
-  __shared__ uint32_t digit_base[16];
-  const int t = threadIdx.x;
-  int32_t* bufk[2] = {const_cast<int32_t*>(a.kin), a.kout};
-  int32_t* bufv[2] = {const_cast<int32_t*>(a.vin), a.vout};
-  uint32_t* wa = words;                          // padded word arrays of one chunk
-  uint32_t* wb = words + kLocalThreads * kLocalPad;
-  for (int pass = 0; pass < 4; ++pass) {
-    const int shift = 4 * pass;
-    const int32_t* sk = bufk[pass & 1];
-    const int32_t* sv = bufv[pass & 1];
-    int32_t* dk = bufk[(pass + 1) & 1];
-    int32_t* dv = bufv[(pass + 1) & 1];
-    // digit counts of the whole bucket, then their exclusive prefix
-    if (t < 16) digit_base[t] = 0;
-    __syncthreads();
-    for (int64_t i = t; i < size; i += kLocalThreads)
-      atomicAdd(&digit_base[(static_cast<uint32_t>(sk[begin + i]) >> shift) & 15u], 1u);
-    __syncthreads();
-    if (t == 0) {
-      uint32_t run = 0;
-      for (int d = 0; d < 16; ++d) {
-        const uint32_t c = digit_base[d];
-        digit_base[d] = run;
-        run += c;
-      }
-    }
-    __syncthreads();
-    for (int64_t c0 = 0; c0 < size; c0 += kLocalCap) {
-      const int cnt = static_cast<int>((size - c0) < kLocalCap ? (size - c0) : kLocalCap);
-      // words of the chunk: (digit << 13) | row within the chunk, in chunk order
-#pragma unroll
-      for (int i = 0; i < kLocalIpt; ++i) {
-        const int p = t * kLocalIpt + i;
-        if (p < cnt) {
-          const uint32_t d = (static_cast<uint32_t>(sk[begin + c0 + p]) >> shift) & 15u;
-          wa[t * kLocalPad + i] = (d << 13) | static_cast<uint32_t>(p);
-        }
-      }
-      __syncthreads();
-      local_pass(wa, wb, cnt, 13, scan, tmp);
-      // wb holds the chunk stably ordered by digit; a word's rank inside its digit is its
-      // position minus the chunk's count of smaller digits
-      __shared__ uint32_t chunk_start[16];
-      __shared__ uint32_t chunk_count[16];
-      if (t < 16) chunk_count[t] = 0;
-      __syncthreads();
-      for (int p = t; p < cnt; p += kLocalThreads) atomicAdd(&chunk_count[wb[padded(p)] >> 13], 1u);
-      __syncthreads();
-      if (t == 0) {
-        uint32_t run = 0;
-        for (int d = 0; d < 16; ++d) {
-          chunk_start[d] = run;
-          run += chunk_count[d];
-        }
-      }
-      __syncthreads();
-      for (int p = t; p < cnt; p += kLocalThreads) {
-        const uint32_t w = wb[padded(p)];
-        const uint32_t d = w >> 13, row = w & 8191u;
-        const int64_t g = begin + digit_base[d] + (p - chunk_start[d]);
-        dk[g] = sk[begin + c0 + row];
-        dv[g] = sv[begin + c0 + row];
-      }
-      __syncthreads();
-      if (t < 16) digit_base[t] += chunk_count[t];
-      __syncthreads();
-    }
-    __threadfence_block();
-    __syncthreads();
-  }
-  // four passes end in kin: copy the bucket to kout
-  for (int64_t i = t; i < size; i += kLocalThreads) {
-    a.kout[begin + i] = a.kin[begin + i];
-    a.vout[begin + i] = a.vin[begin + i];
-  }
-}
-
-__global__ void __launch_bounds__(kLocalThreads) local_sort_kernel(const __grid_constant__ LocalArgs a) {
-  extern __shared__ __align__(16) uint32_t local_smem[];
-  uint32_t* wa = local_smem;                                   // padded words, ping
-  uint32_t* wb = local_smem + kLocalThreads * kLocalPad;      // pong
-  uint32_t* scan = wb + kLocalThreads * kLocalPad;            // 16 x kLocalThreads counters
-  __shared__ uint32_t tmp[kWarp + 1];
-  const int t = threadIdx.x;
-  const int64_t begin = a.bucket_begin[blockIdx.x];
-  const int64_t size = a.bucket_count[blockIdx.x];
-  if (size == 0) return;
-  if (size > kLocalCap) {
-    local_sort_large(a, begin, size, local_smem, scan, tmp);
-    return;
-  }
-  const int cnt = static_cast<int>(size);
-#pragma unroll
-  for (int i = 0; i < kLocalIpt; ++i) {
-    const int p = t * kLocalIpt + i;
-    if (p < cnt) wa[t * kLocalPad + i] = ((static_cast<uint32_t>(a.kin[begin + p]) & 0xFFFFu) << 13) | static_cast<uint32_t>(p);
-  }
-  __syncthreads();
-  local_pass(wa, wb, cnt, 13, scan, tmp);
-  local_pass(wb, wa, cnt, 17, scan, tmp);
-  local_pass(wa, wb, cnt, 21, scan, tmp);
-  local_pass(wb, wa, cnt, 25, scan, tmp);
-  for (int p = t; p < cnt; p += kLocalThreads) {
-    const uint32_t row = wa[padded(p)] & 8191u;
-    a.kout[begin + p] = a.kin[begin + row];
-    a.vout[begin + p] = a.vin[begin + row];
-  }
-}
-
-constexpr size_t kLocalSmem = (2 * kLocalThreads * kLocalPad + 16 * kLocalThreads) * sizeof(uint32_t);
 
 // ---------------------------------------------------------------- partitioned join
 //
@@ -517,7 +339,7 @@ constexpr int kJoinSlots = 8192;                      // 64 KB table in shared m
 struct JoinArgs {
   const int32_t* bkey;  // build side, partitioned
   const int32_t* bval;
-  const int64_t* b_begin;   // [partitions]
+  const uint32_t* b_begin;  // [partitions]
   const uint32_t* b_count;  // [partitions]
   const int32_t* pkey;      // probe side, partitioned
   const int32_t* ppay;
@@ -541,14 +363,14 @@ __device__ __forceinline__ uint32_t slot_hash(int32_t k) {
 }
 
 // The single partition of a join whose build side needs no partitioning.
-__global__ void one_partition_kernel(int64_t nb, int64_t np, int tile_rows, int64_t* b_begin, uint32_t* b_count,
-                                     int64_t* p_begin, int64_t* p_size, uint32_t* p_tiles) {
+__global__ void one_partition_kernel(uint32_t nb, uint32_t np, int rows, uint32_t* b_begin, uint32_t* b_count,
+                                     uint32_t* p_begin, uint32_t* p_size, uint32_t* p_tiles) {
   b_begin[0] = 0;
-  b_count[0] = static_cast<uint32_t>(nb);
+  b_count[0] = nb;
   p_begin[0] = 0;
   p_size[0] = np;
   p_tiles[0] = 0;
-  p_tiles[1] = static_cast<uint32_t>((np + tile_rows - 1) / tile_rows);
+  p_tiles[1] = (np + static_cast<uint32_t>(rows) - 1) / static_cast<uint32_t>(rows);
 }
 
 // Table capacity of a build partition: a power of two of at least twice its rows.
@@ -580,18 +402,27 @@ __device__ __forceinline__ void join_insert(const JoinArgs& a, int64_t bb, uint3
 }
 
 // Build partitions too large for shared memory get their table in the global arena, built
-// once here (one block per partition) before any probe reads it.
+// once here before any probe reads it.  A block looks at one partition per thread and builds
+// the tables of those that are too large, one after the other.
 __global__ void __launch_bounds__(kJoinThreads) join_build_large_kernel(const __grid_constant__ JoinArgs a, int parts) {
-  const int p = blockIdx.x;
-  if (p >= parts) return;
-  const uint32_t bn = a.b_count[p];
-  const uint32_t cap = join_capacity(bn);
-  if (cap <= static_cast<uint32_t>(kJoinSlots)) return;
-  const int64_t bb = a.b_begin[p];
-  uint64_t* table = a.arena + 4 * bb;
-  for (uint32_t i = threadIdx.x; i < cap; i += kJoinThreads) table[i] = kEmptySlot;
+  __shared__ int list[kJoinThreads];
+  __shared__ int found;
+  if (threadIdx.x == 0) found = 0;
   __syncthreads();
-  join_insert(a, bb, bn, table, cap, kJoinThreads);
+  const int mine = static_cast<int>(blockIdx.x) * kJoinThreads + static_cast<int>(threadIdx.x);
+  if (mine < parts && join_capacity(a.b_count[mine]) > static_cast<uint32_t>(kJoinSlots))
+    list[atomicAdd(&found, 1)] = mine;
+  __syncthreads();
+  for (int j = 0; j < found; ++j) {
+    const int p = list[j];
+    const uint32_t bn = a.b_count[p];
+    const uint32_t cap = join_capacity(bn);
+    const int64_t bb = a.b_begin[p];
+    uint64_t* table = a.arena + 4 * bb;
+    for (uint32_t i = threadIdx.x; i < cap; i += kJoinThreads) table[i] = kEmptySlot;
+    __syncthreads();
+    join_insert(a, bb, bn, table, cap, kJoinThreads);
+  }
 }
 
 // Bulk L2 prefetch of rows [row, row + rows) of a column (whole 16-byte groups inside the
@@ -612,20 +443,23 @@ __global__ void __launch_bounds__(kJoinThreads, 2) join_partition_kernel(const _
   const uint32_t t1 = static_cast<uint32_t>((static_cast<uint64_t>(total) * (blockIdx.x + 1)) / gridDim.x);
   uint64_t sum = 0, matches = 0;
   int built = -1;  // partition whose table is in shared memory
+  int p = t0 < t1 ? find_segment(a.probe, t0) : 0;
   for (uint32_t b = t0; b < t1; ++b) {
-    const TileAt at = find_tile(a.probe, b, kJoinTile);
-    const int p = at.seg;
+    while (b >= a.probe.tile_start[p + 1]) ++p;
+    const TileAt at = tile_rows(a.probe, p, b, kJoinTile);
     const int64_t bb = a.b_begin[p];
     const uint32_t bn = a.b_count[p];
     const uint32_t cap = join_capacity(bn);
     const bool in_smem = cap <= static_cast<uint32_t>(kJoinSlots);
     if (tid == 0 && b + 1 < t1) {  // the next tile's rows travel to L2 meanwhile
-      const TileAt nx = find_tile(a.probe, b + 1, kJoinTile);
+      int q = p;
+      while (b + 1 >= a.probe.tile_start[q + 1]) ++q;
+      const TileAt nx = tile_rows(a.probe, q, b + 1, kJoinTile);
       prefetch_rows(a.pkey, nx.row0, nx.valid);
       prefetch_rows(a.ppay, nx.row0, nx.valid);
-      if (nx.seg != p) {
-        prefetch_rows(a.bkey, a.b_begin[nx.seg], a.b_count[nx.seg]);
-        prefetch_rows(a.bval, a.b_begin[nx.seg], a.b_count[nx.seg]);
+      if (q != p) {
+        prefetch_rows(a.bkey, a.b_begin[q], a.b_count[q]);
+        prefetch_rows(a.bval, a.b_begin[q], a.b_count[q]);
       }
     }
     const uint64_t* table = in_smem ? stab : a.arena + 4 * bb;  // the arena's table is built already
@@ -688,45 +522,56 @@ struct Carve {
 
 // Device arrays of one partition level of one side.
 struct Level {
-  int64_t* seg_begin;
-  int64_t* seg_size;
-  uint32_t* tile_start;
-  uint32_t* tile_seg;         // [tiles]
-  uint32_t* hist;             // [segments][256]
-  unsigned long long* cursor;  // [segments][256]
-  int64_t* bucket_begin;      // [segments * 256]
+  uint32_t* seg_begin;     // [segments] (level B: the bucket starts and counts of level A)
+  uint32_t* seg_size;      // [segments]
+  uint32_t* tile_start;    // [segments + 1]
+  uint32_t* hist;          // [segments][digits]
+  uint32_t* cursor;        // [segments][digits], stride words apart
+  int stride;
+  uint32_t* bucket_begin;  // [segments][digits]
 };
 
-int64_t tiles_bound(int64_t n, int segments, int tile_rows) { return (n + tile_rows - 1) / tile_rows + segments; }
+int64_t tiles_bound(int64_t n, int segments, int rows) { return (n + rows - 1) / rows + segments; }
 
-Level carve_level(Carve& c, int segments, int64_t rows) {
+Level carve_level(Carve& c, int segments, int digits) {
+  const size_t buckets = static_cast<size_t>(segments) * digits;
   Level L;
-  L.seg_begin = c.take<int64_t>(segments);
-  L.seg_size = c.take<int64_t>(segments);
+  L.seg_begin = c.take<uint32_t>(segments);
+  L.seg_size = c.take<uint32_t>(segments);
   L.tile_start = c.take<uint32_t>(segments + 1);
-  L.tile_seg = c.take<uint32_t>(static_cast<size_t>(tiles_bound(rows, segments, kPartTile)));
-  L.hist = c.take<uint32_t>(static_cast<size_t>(segments) * kBuckets);
-  L.cursor = c.take<unsigned long long>(static_cast<size_t>(segments) * kBuckets);
-  L.bucket_begin = c.take<int64_t>(static_cast<size_t>(segments) * kBuckets);
+  L.hist = c.take<uint32_t>(buckets);
+  L.stride = segments == 1 ? kCursorStrideA : kCursorStrideB;
+  L.cursor = c.take<uint32_t>(buckets * L.stride);
+  L.bucket_begin = c.take<uint32_t>(buckets);
   return L;
 }
 
 // One partition pass over the segments of L (already set up): histogram, scan, scatter.
-int run_pass(const Level& L, int segments, int64_t n, const int32_t* kin, const int32_t* vin, int32_t* kout,
-             int32_t* vout, DigitFn f, int32_t* err, cudaStream_t s) {
-  if (cudaMemsetAsync(L.hist, 0, static_cast<size_t>(segments) * kBuckets * 4, s) != cudaSuccess) return CRYS_ECUDA;
-  Segs S{L.seg_begin, L.seg_size, L.tile_start, L.tile_seg, segments};
+template <typename Digit>
+int run_pass(const Level& L, int segments, int digits, int64_t n, const int32_t* kin, const int32_t* vin, int32_t* kout,
+             int32_t* vout, Digit f, int32_t* err, cudaStream_t s) {
+  if (cudaMemsetAsync(L.hist, 0, static_cast<size_t>(segments) * digits * 4, s) != cudaSuccess) return CRYS_ECUDA;
+  Segs S{L.seg_begin, L.seg_size, L.tile_start, segments};
   const int64_t grid = tiles_bound(n, segments, kPartTile);
   const int64_t hist_grid = grid < static_cast<int64_t>(sm_count()) * 8 ? grid : static_cast<int64_t>(sm_count()) * 8;
-  part_hist_kernel<<<static_cast<unsigned>(hist_grid), kPartThreads, 0, s>>>(kin, S, f, L.hist);
+  part_hist_kernel<<<static_cast<unsigned>(hist_grid), kHistThreads, 0, s>>>(kin, S, f, digits, L.hist);
   note_launch();
-  part_scan_kernel<<<static_cast<unsigned>(segments), kBuckets, 0, s>>>(L.hist, L.seg_begin, L.cursor,
-                                                                        L.bucket_begin);
+  part_scan_kernel<<<static_cast<unsigned>(segments), kBuckets, 0, s>>>(L.hist, L.seg_begin, digits, L.cursor,
+                                                                        L.stride, L.bucket_begin);
   note_launch();
-  ScatterArgs a{kin, vin, kout, vout, S, f, L.cursor, err};
+  ScatterArgs<Digit> a{kin, vin, kout, vout, S, f, digits, L.cursor, L.stride, err};
   const size_t smem = static_cast<size_t>(kPartTile) * 8;
-  if (!allow_smem(part_scatter_kernel, smem)) return CRYS_ECUDA;
-  part_scatter_kernel<<<static_cast<unsigned>(grid), kPartThreads, smem, s>>>(a);
+  if (!allow_smem(part_scatter_kernel<Digit>, smem)) return CRYS_ECUDA;
+  part_scatter_kernel<Digit><<<static_cast<unsigned>(grid), kPartThreads, smem, s>>>(a);
+  note_launch();
+  return check_launch();
+}
+
+// The buckets of level A as the segments of level B.
+int next_level(const Level& A, Level& B, int segments, cudaStream_t s) {
+  B.seg_begin = A.bucket_begin;
+  B.seg_size = A.hist;
+  tile_prefix_kernel<<<1, 1024, 0, s>>>(A.hist, segments, kPartTile, B.tile_start);
   note_launch();
   return check_launch();
 }
@@ -753,18 +598,22 @@ extern "C" int crys_sort_msb(const int32_t* keys_in, const int32_t* vals_in, int
                              int64_t n, void* d_temp, size_t* temp_bytes, crys_stream stream) {
   using namespace crys;
   if (n < 0 || n > (1ll << 31) - 1) return CRYS_EINVAL;
-  // scratch: a (key, value) buffer of n rows and the two levels' arrays
-  auto layout = [&](void* base, int32_t** tk, int32_t** tv, Level* A, Level* B) {
+  const int bits = range_bits(n, kLocalCap);
+  const int b2 = bits > 8 ? bits - 8 : 0, digits2 = 1 << b2;
+  // scratch: a (key, value) buffer of n rows, the key range and the two levels' arrays
+  auto layout = [&](void* base, int32_t** tk, int32_t** tv, KeyRange** range, Level* A, Level* B) {
     Carve c(base);
     *tk = c.take<int32_t>(static_cast<size_t>(n));
     *tv = c.take<int32_t>(static_cast<size_t>(n));
-    *A = carve_level(c, 1, n);
-    *B = carve_level(c, kBuckets, n);
+    *range = c.take<KeyRange>(1);
+    *A = carve_level(c, 1, kBuckets);
+    *B = carve_level(c, kBuckets, digits2);
     return c.off;
   };
   int32_t *tk, *tv;
+  KeyRange* range;
   Level A, B;
-  const size_t need = layout(nullptr, &tk, &tv, &A, &B);
+  const size_t need = layout(nullptr, &tk, &tv, &range, &A, &B);
   if (!d_temp && temp_bytes) {
     *temp_bytes = need;
     return CRYS_OK;
@@ -778,27 +627,33 @@ extern "C" int crys_sort_msb(const int32_t* keys_in, const int32_t* vals_in, int
       !no_overlap(vals_out, nb, keys_in, nb) || !no_overlap(vals_out, nb, vals_in, nb) ||
       !no_overlap(keys_out, nb, vals_out, nb))
     return CRYS_EINVAL;
-  layout(d_temp, &tk, &tv, &A, &B);
+  layout(d_temp, &tk, &tv, &range, &A, &B);
   int32_t* err = device_error_word();
   if (!err) return CRYS_ECUDA;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  // level A: the whole array by the top digit (sign bit flipped), input -> output buffers
-  seg_init_kernel<<<1, 1, 0, s>>>(n, kPartTile, A.seg_begin, A.seg_size, A.tile_start);
+  const uint32_t rows = static_cast<uint32_t>(n);
+  if (bits == 0)  // one block sorts everything
+    return launch_local_sort<false>(LocalArgs{keys_in, vals_in, keys_out, vals_out, nullptr, nullptr, rows, err}, 1, s);
+  if (launch_key_range(keys_in, n, bits, range, s) != CRYS_OK) return CRYS_ECUDA;
+  // level A: the whole array by the leading 8 bits
+  seg_init_kernel<<<1, 1, 0, s>>>(rows, kPartTile, A.seg_begin, A.seg_size, A.tile_start);
   note_launch();
-  int rc = run_pass(A, 1, n, keys_in, vals_in, keys_out, vals_out, DigitFn{1u, 24u, 0xFFu, 0x80u}, err, s);
+  int32_t* ak = b2 ? keys_out : tk;
+  int32_t* av = b2 ? vals_out : tv;
+  int rc = run_pass(A, 1, kBuckets, n, keys_in, vals_in, ak, av, RangeDigit{range, static_cast<uint32_t>(b2), 0xFFu}, err, s);
   if (rc != CRYS_OK) return rc;
-  // level B: each of the 256 buckets by the next digit, output -> scratch buffers
-  seg_from_buckets_kernel<<<1, 1024, 0, s>>>(A.bucket_begin, A.hist, kBuckets, kPartTile, B.seg_begin, B.seg_size,
-                                             B.tile_start, B.tile_seg);
-  note_launch();
-  rc = run_pass(B, kBuckets, n, keys_out, vals_out, tk, tv, DigitFn{1u, 16u, 0xFFu, 0u}, err, s);
-  if (rc != CRYS_OK) return rc;
-  // every bucket of the top 16 bits sorted by the low 16 bits, scratch -> output
-  LocalArgs L{tk, tv, keys_out, vals_out, B.bucket_begin, B.hist, err};
-  if (!allow_smem(local_sort_kernel, kLocalSmem)) return CRYS_ECUDA;
-  local_sort_kernel<<<kBuckets * kBuckets, kLocalThreads, kLocalSmem, s>>>(L);
-  note_launch();
-  return check_launch();
+  const Level* last = &A;
+  if (b2) {
+    // level B: each of the 256 buckets by the next bits, output -> scratch buffers
+    rc = next_level(A, B, kBuckets, s);
+    if (rc != CRYS_OK) return rc;
+    rc = run_pass(B, kBuckets, digits2, n, ak, av, tk, tv, RangeDigit{range, 0u, static_cast<uint32_t>(digits2 - 1)}, err, s);
+    if (rc != CRYS_OK) return rc;
+    last = &B;
+  }
+  // every bucket sorted by its remaining bits, scratch -> output
+  return launch_local_sort<true>(LocalArgs{tk, tv, keys_out, vals_out, last->bucket_begin, last->hist, rows, err},
+                                 static_cast<unsigned>(1u << bits), s);
 }
 
 extern "C" int crys_join_partitioned(const int32_t* bkeys, const int32_t* bvals, int64_t nb, const int32_t* fk,
@@ -809,20 +664,18 @@ extern "C" int crys_join_partitioned(const int32_t* bkeys, const int32_t* bvals,
   const int bits = join_bits(nb);
   const int b1 = (bits + 1) / 2, b2 = bits / 2;
   const int parts1 = 1 << b1;
-  // partition index space: bucket d of pass-2 segment g is partition g * 256 + d (digits
-  // of a narrower pass leave the upper buckets empty)
-  const int parts = bits == 0 ? 1 : (b2 == 0 ? kBuckets : parts1 * kBuckets);
+  // bucket d of pass-2 segment g is partition (g << b2) + d
+  const int parts = 1 << bits;
   struct Side {
     int32_t *k1, *v1, *k2, *v2;  // rows after pass 1 and after pass 2
     Level A, B;
   };
   struct Parts {  // the partitions the join kernel reads
-    int64_t* b_begin;
+    uint32_t* b_begin;
     uint32_t* b_count;
-    int64_t* p_begin;
-    int64_t* p_size;
+    uint32_t* p_begin;
+    uint32_t* p_size;
     uint32_t* p_tiles;
-    uint32_t* p_tile_seg;
     uint64_t* arena;
   };
   auto layout = [&](void* base, Side* R, Side* P, Parts* J) {
@@ -833,15 +686,14 @@ extern "C" int crys_join_partitioned(const int32_t* bkeys, const int32_t* bvals,
       sd->v1 = c.take<int32_t>(rows);
       sd->k2 = c.take<int32_t>(rows);
       sd->v2 = c.take<int32_t>(rows);
-      sd->A = carve_level(c, 1, static_cast<int64_t>(rows));
-      sd->B = carve_level(c, parts1, static_cast<int64_t>(rows));
+      sd->A = carve_level(c, 1, parts1);
+      sd->B = carve_level(c, parts1, 1 << b2);
     }
-    J->b_begin = c.take<int64_t>(1);
+    J->b_begin = c.take<uint32_t>(1);
     J->b_count = c.take<uint32_t>(1);
-    J->p_begin = c.take<int64_t>(static_cast<size_t>(parts));
-    J->p_size = c.take<int64_t>(static_cast<size_t>(parts));
+    J->p_begin = c.take<uint32_t>(1);
+    J->p_size = c.take<uint32_t>(1);
     J->p_tiles = c.take<uint32_t>(static_cast<size_t>(parts) + 1);
-    J->p_tile_seg = c.take<uint32_t>(static_cast<size_t>(tiles_bound(np, parts, kJoinTile)));
     J->arena = c.take<uint64_t>(static_cast<size_t>(4) * static_cast<size_t>(nb > 0 ? nb : 1));
     return c.off;
   };
@@ -865,47 +717,49 @@ extern "C" int crys_join_partitioned(const int32_t* bkeys, const int32_t* bvals,
   if (!err) return CRYS_ECUDA;
   // both sides partitioned by the same hash bits: pass 1 by the top b1 bits, pass 2 by
   // the next b2 bits inside each pass-1 partition
-  const DigitFn f1{2654435769u, static_cast<uint32_t>(32 - b1), static_cast<uint32_t>(parts1 - 1), 0u};
-  const DigitFn f2{2654435769u, static_cast<uint32_t>(32 - bits), static_cast<uint32_t>((1 << b2) - 1), 0u};
+  const HashDigit f1{static_cast<uint32_t>(32 - b1), static_cast<uint32_t>(parts1 - 1)};
+  const HashDigit f2{static_cast<uint32_t>(32 - bits), static_cast<uint32_t>((1 << b2) - 1)};
   Side* sides[2] = {&R, &P};
   const int32_t* in_k[2] = {bkeys, fk};
   const int32_t* in_v[2] = {bvals, payload};
   const int64_t rows[2] = {nb, np};
   const int32_t* fin_k[2] = {bkeys, fk};
   const int32_t* fin_v[2] = {bvals, payload};
-  const int64_t* fin_begin[2] = {nullptr, nullptr};
+  const uint32_t* fin_begin[2] = {nullptr, nullptr};
   const uint32_t* fin_count[2] = {nullptr, nullptr};
   for (int w = 0; w < 2 && bits > 0; ++w) {
     Side& sd = *sides[w];
-    seg_init_kernel<<<1, 1, 0, s>>>(rows[w], kPartTile, sd.A.seg_begin, sd.A.seg_size, sd.A.tile_start);
+    seg_init_kernel<<<1, 1, 0, s>>>(static_cast<uint32_t>(rows[w]), kPartTile, sd.A.seg_begin, sd.A.seg_size, sd.A.tile_start);
     note_launch();
-    int rc = run_pass(sd.A, 1, rows[w], in_k[w], in_v[w], sd.k1, sd.v1, f1, err, s);
+    int rc = run_pass(sd.A, 1, parts1, rows[w], in_k[w], in_v[w], sd.k1, sd.v1, f1, err, s);
     if (rc != CRYS_OK) return rc;
     fin_k[w] = sd.k1;
     fin_v[w] = sd.v1;
     fin_begin[w] = sd.A.bucket_begin;
     fin_count[w] = sd.A.hist;
     if (b2 == 0) continue;
-    seg_from_buckets_kernel<<<1, 1024, 0, s>>>(sd.A.bucket_begin, sd.A.hist, parts1, kPartTile, sd.B.seg_begin,
-                                               sd.B.seg_size, sd.B.tile_start, sd.B.tile_seg);
-    note_launch();
-    rc = run_pass(sd.B, parts1, rows[w], sd.k1, sd.v1, sd.k2, sd.v2, f2, err, s);
+    rc = next_level(sd.A, sd.B, parts1, s);
+    if (rc != CRYS_OK) return rc;
+    rc = run_pass(sd.B, parts1, 1 << b2, rows[w], sd.k1, sd.v1, sd.k2, sd.v2, f2, err, s);
     if (rc != CRYS_OK) return rc;
     fin_k[w] = sd.k2;
     fin_v[w] = sd.v2;
     fin_begin[w] = sd.B.bucket_begin;
     fin_count[w] = sd.B.hist;
   }
-  const int64_t* b_begin = fin_begin[0];
+  const uint32_t* b_begin = fin_begin[0];
   const uint32_t* b_count = fin_count[0];
+  const uint32_t* p_begin = fin_begin[1];
+  const uint32_t* p_size = fin_count[1];
   if (bits == 0) {  // one partition: the inputs as they are
-    one_partition_kernel<<<1, 1, 0, s>>>(nb, np, kJoinTile, J.b_begin, J.b_count, J.p_begin, J.p_size, J.p_tiles);
+    one_partition_kernel<<<1, 1, 0, s>>>(static_cast<uint32_t>(nb), static_cast<uint32_t>(np), kJoinTile, J.b_begin, J.b_count, J.p_begin, J.p_size, J.p_tiles);
     note_launch();
     b_begin = J.b_begin;
     b_count = J.b_count;
+    p_begin = J.p_begin;
+    p_size = J.p_size;
   } else {
-    seg_from_buckets_kernel<<<1, 1024, 0, s>>>(fin_begin[1], fin_count[1], parts, kJoinTile, J.p_begin, J.p_size,
-                                               J.p_tiles, J.p_tile_seg);
+    tile_prefix_kernel<<<1, 1024, 0, s>>>(fin_count[1], parts, kJoinTile, J.p_tiles);
     note_launch();
   }
   JoinArgs a;
@@ -915,12 +769,12 @@ extern "C" int crys_join_partitioned(const int32_t* bkeys, const int32_t* bvals,
   a.b_count = b_count;
   a.pkey = fin_k[1];
   a.ppay = fin_v[1];
-  a.probe = Segs{J.p_begin, J.p_size, J.p_tiles, J.p_tile_seg, parts};
+  a.probe = Segs{p_begin, p_size, J.p_tiles, parts};
   a.arena = J.arena;
   a.sum = reinterpret_cast<unsigned long long*>(d_sum);
   a.matches = reinterpret_cast<unsigned long long*>(d_matches);
   a.err = err;
-  join_build_large_kernel<<<static_cast<unsigned>(parts), kJoinThreads, 0, s>>>(a, parts);
+  join_build_large_kernel<<<static_cast<unsigned>((parts + kJoinThreads - 1) / kJoinThreads), kJoinThreads, 0, s>>>(a, parts);
   note_launch();
   const size_t smem = static_cast<size_t>(kJoinSlots) * 8;
   if (!allow_smem(join_partition_kernel, smem)) return CRYS_ECUDA;
