@@ -191,10 +191,13 @@ int crys_probe_aggregate(const int32_t* fk, const int32_t* payload, int64_t n,
                          crys_stream s);
 
 /* ------------------------------------------------------------------ sort
- * Section 4.4: least-significant-digit radix sort of (key, value) pairs by signed int32
- * key, 8-bit digits, 4 passes, stable.  One up-front pass histograms all four digits;
- * each digit pass ranks a tile stably inside the thread block and finds the tile's
- * output offsets with a chained (decoupled look-back) scan.  n <= 2^30 - 1.
+ * Section 4.4: stable radix sort of (key, value) pairs by signed int32 key with 8-bit
+ * stable passes.  Keys that spread evenly enough over their range take at most two passes, by
+ * the leading bits of a key's place in the range, and every bucket of about 4096 rows is
+ * then sorted inside one thread block; other keys take a least-significant-digit sort, a
+ * pass per 8-bit digit that varies.  The choice is made on the device.  Each pass ranks a
+ * tile stably inside the thread block and finds the tile's output offsets with a chained
+ * scan over the tiles.  Up to 4992 rows are sorted by one block.  n <= 2^30 - 1.
  * keys_out/vals_out must not overlap the inputs; the inputs are not modified. */
 int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out,
               int32_t* vals_out, int64_t n, void* d_temp, size_t* temp_bytes, crys_stream s);

@@ -94,6 +94,26 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   }
 }
 
+// Bookkeeping of one spin-wait on a word that another block of the same launch writes: false once
+// the wait's bound has passed (CRYS_DEV_TIMEOUT and the call's abort word are set) or
+// another block of the call gave up (its abort word, in the call's scratch: a failure of an
+// earlier call does not reach this one).  Looks only every 32nd time.
+struct SpinGuard {
+  uint64_t t0 = 0;
+  uint32_t spins = 0;
+  __device__ __forceinline__ bool go_on(unsigned int* abort_word, uint64_t wait_ns, int32_t* err) {
+    if (++spins % 32 != 0) return true;
+    const uint64_t now = global_timer_ns();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > wait_ns) {
+      set_error(err, CRYS_DEV_TIMEOUT);
+      *reinterpret_cast<volatile unsigned int*>(abort_word) = 1u;
+      return false;
+    }
+    return *reinterpret_cast<volatile unsigned int*>(abort_word) == 0u;
+  }
+};
+
 // L2 eviction policies for bulk copies and loads: streamed columns are read once
 // (evict_first) so that hash tables probed at random stay resident (evict_last).
 __device__ __forceinline__ uint64_t policy_evict_first() {

@@ -249,25 +249,6 @@ struct OrderedShared {
   uint32_t ticket;             // 0: this block is the scanner
 };
 
-// One waiting warp's bookkeeping: false once the wait's bound has passed or another block of
-// this call gave up (its abort word, in this call's scratch: a failure of an earlier call
-// does not reach this one).  Looks only every 32nd time.
-struct SpinGuard {
-  uint64_t t0 = 0;
-  uint32_t spins = 0;
-  __device__ __forceinline__ bool go_on(const SelectArgs& a) {
-    if (++spins % 32 != 0) return true;
-    const uint64_t now = global_timer_ns();
-    if (t0 == 0) t0 = now;
-    if (now - t0 > a.wait_ns) {
-      set_error(a.err, CRYS_DEV_TIMEOUT);
-      st_relaxed_u32(a.abort_word, 1u);
-      return false;
-    }
-    return ld_relaxed_u32(a.abort_word) == 0u;
-  }
-};
-
 // The scanner: warp w of the block takes the chunks w, w + WARPS, ... of kChunk status words,
 // reads each until it is published and, once the earlier chunks are done, hands out
 // positions to the published words in front of the first missing one.  (Not only to whole
@@ -309,7 +290,7 @@ __device__ void scan_tiles(const SelectArgs& a, OrderedShared& sh, int64_t ntile
       }
       const bool mine = __shfl_sync(0xFFFFFFFFu, static_cast<int>(*turn == c), 0) != 0;
       if (there == handed || !mine) {
-        if (!__all_sync(0xFFFFFFFFu, guard.go_on(a)) || __any_sync(0xFFFFFFFFu, *gave_up)) {
+        if (!__all_sync(0xFFFFFFFFu, guard.go_on(a.abort_word, a.wait_ns, a.err)) || __any_sync(0xFFFFFFFFu, *gave_up)) {
           if (lane == 0) *gave_up = 1;
           return;
         }
@@ -417,7 +398,7 @@ __global__ void __launch_bounds__(THREADS + 2 * kWarp) select_ordered_kernel(Sel
         const uint64_t* word = &a.tile_state[sh.tile[s]];
         SpinGuard guard;
         uint64_t w = ld_relaxed_u64(word);
-        while ((w >> 62) != 2u && guard.go_on(a)) w = ld_relaxed_u64(word);
+        while ((w >> 62) != 2u && guard.go_on(a.abort_word, a.wait_ns, a.err)) w = ld_relaxed_u64(word);
         if ((w >> 62) == 2u) base = static_cast<long long>(w & kValueMask);
         if (base >= 0 && base + ttot[s] > a.n) {
           set_error(a.err, CRYS_DEV_BOUNDS);

@@ -1,24 +1,32 @@
-// Least-significant-digit radix sort of (key, value) pairs (Section 4.4): 8-bit digits,
-// four stable radix-partition passes from the low digit to the high digit.
+// Stable radix sort of (key, value) pairs (Section 4.4), by signed key.
 //
-// The paper's passes each run a histogram phase and a shuffle phase; here
-//  * one up-front kernel reads the keys once and histograms all four digits (the
-//    global start of every digit bucket of every pass, after a 256-wide scan), and
-//  * each pass is ONE kernel: a thread block takes the next tile id from an atomic
-//    counter, ranks its keys stably inside the block (per-warp multisplit with
-//    ballots: keys are processed warp-striped, round by round, so rank order equals
-//    input order), publishes its per-digit counts and finds the counts of all earlier tiles
-//    with a decoupled look-back, then writes keys and values through shared memory in
-//    sorted order so that each digit's run is stored with consecutive addresses.
-// So the data crosses HBM once per pass (read 8N, write 8N) plus one 4N key read.
+// Two plans, chosen on the device from the keys:
+//  * buckets: the keys are spread over up to 2^16 buckets of about 4096 rows by their leading
+//    bits - one stable radix pass of 8 bits, or two, low bits first - and every bucket is
+//    then sorted inside one thread block (localsort.cuh).  The leading bits are those of a
+//    key's place between the smallest and largest key of a sample (keyrange.cuh), so narrow
+//    ranges fill the buckets too.  One kernel reads the keys and counts all buckets, which
+//    gives the passes' bucket starts and shows whether any bucket is too large for a block.
+//  * digits: when one is (heavily repeated or clustered keys), or there are too many rows, the
+//    least-significant-digit sort: 8-bit digits, a stable pass per digit from the low one to
+//    the high one.  Digits that have one value in all keys are skipped.
+//
+// A pass is ONE kernel: a thread block takes the next tile id from an atomic counter, ranks
+// its keys stably inside the block (per-warp multisplit: keys are processed warp-striped,
+// round by round, so rank order equals input order), publishes its per-digit counts, places
+// keys and values in shared memory in sorted order while scanner blocks turn all tiles'
+// counts into positions, and stores each digit's run with consecutive addresses.  So a
+// pass reads 8N and writes 8N.
 //
 // The paper notes that its V100 kernels could partition only 7 bits per stable pass
 // because each thread kept a 2^r histogram in registers; the per-warp shared-memory
-// multisplit used here keeps 8-bit stable passes.  Signed order: the top digit has its
-// sign bit flipped.
-#include <type_traits>
-
+// multisplit used here keeps 8-bit stable passes.
+//
+// 2^28 random pairs: 4.62 ms by buckets (0.2 ms counting, two passes of 1.28 ms, 1.77 ms in
+// the blocks).  Four passes by digits, each with a decoupled look-back, took 6.10 ms.
 #include "common.cuh"
+#include "keyrange.cuh"
+#include "localsort.cuh"
 #include "pipeline.cuh"
 #include "tiles.h"
 
@@ -30,20 +38,176 @@ constexpr int kPasses = 4;
 constexpr uint32_t kFlagAggregate = 1u << 30;
 constexpr uint32_t kFlagInclusive = 2u << 30;
 constexpr uint32_t kValueMask = (1u << 30) - 1;
+// Largest sort by buckets: 2^16 buckets of 4096 rows on average.
+constexpr int64_t kMaxBucketRows = int64_t{4096} << 16;
 
 __device__ __forceinline__ uint32_t digit_of(int32_t key, int pass) {
   const uint32_t d = (static_cast<uint32_t>(key) >> (8 * pass)) & 0xFFu;
   return pass == kPasses - 1 ? d ^ 0x80u : d;
 }
 
-// ---------------------------------------------------------------- histogram
+// What the passes do, written on the device; one per sort, in its scratch.
+struct SortHead {
+  unsigned int tile_counter[kPasses];
+  unsigned int abort_word;   // set by the first block of this sort that gives up
+  unsigned int counted;      // blocks of the counting kernels that have finished
+  unsigned int digits_counted;
+  unsigned int crowded;      // a bucket is too large for a block
+  uint32_t buckets;          // 1: sorted by buckets, 0: by digits
+  uint32_t passes;           // passes that do work; pass j writes to the output when an even number follows
+  KeyRange range;
+  uint32_t shift[kPasses], mask[kPasses];  // a pass's digit
+};
+static_assert(sizeof(SortHead) <= 256, "the head has 256 bytes of the scratch");
+
+// A pass's digit of a key: bits of its place in the key range, or of the key itself with the
+// sign bit flipped.
+template <bool PLACE>
+struct PassDigit {
+  KeyRange range;
+  uint32_t shift, mask;
+  __device__ __forceinline__ uint32_t operator()(int32_t k) const {
+    const uint32_t x = PLACE ? range.place(k) : static_cast<uint32_t>(k) ^ 0x80000000u;
+    return (x >> shift) & mask;
+  }
+};
+
+// ---------------------------------------------------------------- counting the buckets
+
+constexpr int kCountThreads = 1024;
+
+// Exclusive prefix of 256 values held in shared memory, by the first 8 warps of the block.
+__device__ __forceinline__ void scan256(const uint32_t* in, uint32_t* out, uint32_t* tmp) {
+  const int tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
+  uint32_t inc = 0;
+  if (tid < kRadix) {
+    inc = static_cast<uint32_t>(warp_inclusive_scan(static_cast<int32_t>(in[tid]), lane));
+    if (lane == kWarp - 1) tmp[warp] = inc;
+  }
+  __syncthreads();
+  if (tid < kRadix) {
+    uint32_t base = 0;
+    for (int w = 0; w < warp; ++w) base += tmp[w];
+    out[tid] = base + inc - in[tid];
+  }
+  __syncthreads();
+}
+
+// Rows per bucket.  Every block counts its share of the keys in shared memory, two 16-bit
+// counters per word, and stops as soon as one of its buckets is too large for a block (which
+// also keeps the counters from running over: at most 16 more rows per thread follow).  The
+// block that finishes last turns the counts into the passes' bucket starts and the buckets'
+// first rows.
+__global__ void __launch_bounds__(kCountThreads, 1) count_buckets_kernel(const int32_t* __restrict__ keys, int64_t n, int bits,
+                                                                         SortHead* head, uint32_t* counts,
+                                                                         uint32_t* bucket_begin, uint32_t* base) {
+  extern __shared__ __align__(16) uint32_t bins[];  // 2^bits 16-bit counters
+  __shared__ uint32_t col[kRadix], row[kRadix], scanned[kRadix], tmp[kRadix / kWarp];
+  __shared__ unsigned int ticket;
+  const int tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
+  const int words = 1 << (bits - 1);
+  for (int i = tid; i < words; i += kCountThreads) bins[i] = 0;
+  const KeyRange range = head->range;
+  const uint64_t pol = policy_evict_first();
+  __syncthreads();
+  bool over = false;
+  auto add = [&](int32_t k) {
+    const uint32_t b = range.place(k), half = 16u * (b & 1u);
+    over |= ((atomicAdd(&bins[b >> 1], 1u << half) >> half) & 0xFFFFu) >= static_cast<uint32_t>(kLocalCap);
+  };
+  const int64_t nvec = n / 4;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * kCountThreads;
+  int64_t v = static_cast<int64_t>(blockIdx.x) * kCountThreads + tid;
+  volatile unsigned int* crowded = &head->crowded;
+  constexpr int kVecs = 4;  // in flight per thread
+  for (int step = 0; v < nvec && !over; ++step, v += kVecs * stride) {
+    if (step % 8 == 7 && *crowded) break;
+    int4 q[kVecs];
+#pragma unroll
+    for (int j = 0; j < kVecs; ++j)
+      if (v + j * stride < nvec) q[j] = ld_stream_v4(keys + 4 * (v + j * stride), pol);
+#pragma unroll
+    for (int j = 0; j < kVecs; ++j)
+      if (v + j * stride < nvec) {
+        add(q[j].x);
+        add(q[j].y);
+        add(q[j].z);
+        add(q[j].w);
+      }
+  }
+  if (blockIdx.x == 0 && 4 * nvec + tid < n) add(keys[4 * nvec + tid]);  // the last 0..3 keys
+  if (over) *crowded = 1;
+  __syncthreads();
+  if (!*crowded) {
+    for (int i = tid; i < words; i += kCountThreads) {
+      const uint32_t w = bins[i];
+      if (w & 0xFFFFu) atomicAdd(&counts[2 * i], w & 0xFFFFu);
+      if (w >> 16) atomicAdd(&counts[2 * i + 1], w >> 16);
+    }
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) ticket = atomicAdd(&head->counted, 1u);
+  __syncthreads();
+  if (ticket != gridDim.x - 1) return;
+  __threadfence();
+  // the last block: 256 buckets per row (the second pass's digit), one warp per row
+  const int rows = bits > 8 ? 1 << (bits - 8) : 1;
+  if (tid < kRadix) col[tid] = row[tid] = 0;
+  __syncthreads();
+  uint32_t most = 0;
+  for (int r = warp; r < rows; r += kCountThreads / kWarp) {
+    uint32_t sum = 0;
+#pragma unroll
+    for (int j = 0; j < kRadix / kWarp; ++j) {
+      const uint32_t c = __ldcg(&counts[r * kRadix + j * kWarp + lane]);
+      most = max(most, c);
+      sum += c;
+      if (c) atomicAdd(&col[j * kWarp + lane], c);
+    }
+    sum = __reduce_add_sync(0xFFFFFFFFu, sum);
+    if (lane == 0) row[r] = sum;
+  }
+  if (__syncthreads_or(most > static_cast<uint32_t>(kLocalCap) || *crowded != 0)) return;  // head->buckets stays 0
+  scan256(col, scanned, tmp);
+  if (tid < kRadix) base[tid] = scanned[tid];
+  __syncthreads();
+  scan256(row, scanned, tmp);
+  if (tid < kRadix && rows > 1) base[kRadix + tid] = scanned[tid];
+  for (int r = warp; r < rows; r += kCountThreads / kWarp) {
+    uint32_t run = scanned[r];
+#pragma unroll
+    for (int j = 0; j < kRadix / kWarp; ++j) {
+      const uint32_t c = __ldcg(&counts[r * kRadix + j * kWarp + lane]);
+      const uint32_t inc = static_cast<uint32_t>(warp_inclusive_scan(static_cast<int32_t>(c), lane));
+      bucket_begin[r * kRadix + j * kWarp + lane] = run + inc - c;
+      run += __shfl_sync(0xFFFFFFFFu, inc, kWarp - 1);
+    }
+  }
+  if (tid == 0) {
+    head->buckets = 1;
+    head->passes = rows > 1 ? 2 : 1;
+    head->shift[0] = 0;
+    head->mask[0] = kRadix - 1;
+    head->shift[1] = 8;
+    head->mask[1] = static_cast<uint32_t>(rows - 1);
+  }
+}
+
+// ---------------------------------------------------------------- counting the digits
 
 constexpr int kHistThreads = 512;
 constexpr int kHistCopies = 4;  // shared-memory copies of the 4x256 histogram
 
+// Rows per value of every digit; the block that finishes last turns them into the passes'
+// bucket starts.  Nothing to do when the sort goes by buckets.
 __global__ void __launch_bounds__(kHistThreads) sort_hist_kernel(const int32_t* __restrict__ keys,
-                                                                  int64_t n, unsigned int* hist) {
+                                                                  int64_t n, unsigned int* hist, SortHead* head,
+                                                                  uint32_t* base) {
   __shared__ unsigned int h[kHistCopies][kPasses * kRadix];
+  __shared__ unsigned int ticket;
+  __shared__ int varies[kPasses];
+  if (head->buckets) return;
   for (int i = threadIdx.x; i < kHistCopies * kPasses * kRadix; i += kHistThreads)
     (&h[0][0])[i] = 0;
   __syncthreads();
@@ -73,224 +237,348 @@ __global__ void __launch_bounds__(kHistThreads) sort_hist_kernel(const int32_t* 
     for (int r = 0; r < kHistCopies; ++r) c += h[r][i];
     if (c) atomicAdd(hist + i, c);
   }
-}
-
-// Exclusive scan of each pass's 256 digit counts: warp p scans pass p.
-__global__ void sort_scan_kernel(const unsigned int* hist, unsigned int* base) {
-  const int lane = threadIdx.x % kWarp, pass = threadIdx.x / kWarp;
-  if (pass >= kPasses) return;
-  unsigned int carry = 0;
-  for (int c0 = 0; c0 < kRadix; c0 += kWarp) {
-    const unsigned int x = hist[pass * kRadix + c0 + lane];
-    const unsigned int inc = static_cast<unsigned int>(warp_inclusive_scan(static_cast<int32_t>(x), lane));
-    base[pass * kRadix + c0 + lane] = carry + inc - x;
-    carry += __shfl_sync(0xFFFFFFFFu, inc, kWarp - 1);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) ticket = atomicAdd(&head->digits_counted, 1u);
+  __syncthreads();
+  if (ticket != gridDim.x - 1) return;
+  __threadfence();
+  // warp p: does digit p vary, and the starts of its values
+  const int lane = threadIdx.x % kWarp, p = threadIdx.x / kWarp;
+  if (p < kPasses) {
+    bool all = false;
+    for (int c0 = 0; c0 < kRadix; c0 += kWarp) all |= __ldcg(&hist[p * kRadix + c0 + lane]) == static_cast<uint32_t>(n);
+    const bool constant = __any_sync(0xFFFFFFFFu, all) != 0;
+    if (lane == 0) varies[p] = !constant;
   }
+  __syncthreads();
+  int passes = 0;
+  for (int q = 0; q < kPasses; ++q) passes += varies[q];
+  if (p < kPasses && (varies[p] || (passes == 0 && p == 0))) {  // (one key value: one pass copies the rows)
+    int slot = 0;
+    for (int q = 0; q < p; ++q) slot += varies[q];
+    unsigned int carry = 0;
+    for (int c0 = 0; c0 < kRadix; c0 += kWarp) {
+      const unsigned int x = __ldcg(&hist[p * kRadix + c0 + lane]);
+      const unsigned int inc = static_cast<unsigned int>(warp_inclusive_scan(static_cast<int32_t>(x), lane));
+      base[slot * kRadix + c0 + lane] = carry + inc - x;
+      carry += __shfl_sync(0xFFFFFFFFu, inc, kWarp - 1);
+    }
+    if (lane == 0) {
+      head->shift[slot] = static_cast<uint32_t>(8 * p);
+      head->mask[slot] = kRadix - 1;
+    }
+  }
+  if (threadIdx.x == 0) head->passes = passes ? passes : 1;
 }
 
 // ---------------------------------------------------------------- one pass
 
 struct PassArgs {
-  const int32_t* keys_in;
-  const int32_t* vals_in;
-  int32_t* keys_out;
-  int32_t* vals_out;
+  const int32_t *keys_in, *vals_in;  // the sort's input, scratch and output columns
+  int32_t *keys_tmp, *vals_tmp;
+  int32_t *keys_out, *vals_out;
   int64_t n;
   int pass;
+  SortHead* head;
   const unsigned int* digit_base;  // 256 bucket starts of this pass
   uint32_t* status;                // per tile x digit look-back words
-  unsigned int* tile_counter;
-  unsigned int* abort_word;        // set by the first block of this sort that gives up
   uint32_t tile_base;              // first tile id handed out (0 unless a test stalls)
   uint64_t wait_ns;                // bound of a look-back wait
   int32_t* err;
 };
 
-template <int THREADS, int ITEMS, int PASS>
-__global__ void __launch_bounds__(THREADS) sort_pass_kernel(PassArgs a) {
-  constexpr int WARPS = THREADS / kWarp;
-  constexpr int TILE = THREADS * ITEMS;
-  constexpr int WSEG = kWarp * ITEMS;
-  static_assert(THREADS >= kRadix, "one thread per digit");
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  int32_t* skeys = reinterpret_cast<int32_t*>(smem_raw);  // tile keys: input order, then sorted
-  int32_t* svals = skeys + TILE;                           // tile values: input order, then sorted
-  __shared__ unsigned int whist[WARPS][kRadix];  // per-warp digit counts, then offsets
-  __shared__ unsigned int tile_start[kRadix];    // tile-local start of each digit run
-  __shared__ int32_t out_shift[kRadix];          // global position minus local position
-  __shared__ unsigned int scan_tmp[kRadix / kWarp];
-  __shared__ unsigned int tile_sh;
-  __shared__ __align__(8) uint64_t loaded;
+// Columns of one pass.
+struct PassCols {
+  const int32_t *kin, *vin;
+  int32_t *kout, *vout;
+};
 
-  const int tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
-  if (tid == 0) {
-    // a sort whose earlier pass gave up does no further work (tile id past the end)
-    tile_sh = ld_relaxed_u32(a.abort_word) ? 0xFFFFFFFFu : a.tile_base + atomicAdd(a.tile_counter, 1u);
-    mbar_init(&loaded, 1);
-    fence_barrier_init();
+template <int THREADS>
+struct PassShared {
+  alignas(4) uint16_t whist[THREADS / kWarp][kRadix];  // per-warp digit counts, then offsets
+  uint32_t tile_start[kRadix];              // tile-local start of each digit run
+  uint32_t out_shift[kRadix];               // global position minus local position (mod 2^32)
+  uint32_t scan_tmp[kRadix / kWarp];
+  uint32_t tile;
+};
+
+// The scanners: kScanners blocks, the first of a pass to start, turn the tiles' digit counts
+// into exclusive prefixes over the tiles, 32 digits each (one per lane).  Warp w takes the
+// chunks w, w + WARPS, ... of kScanTiles tiles, reads each count until it is published and,
+// once the earlier chunks are done, hands out the prefixes of the published tiles in front
+// of the first missing one.
+//
+// A decoupled look-back, where every tile's block reads earlier tiles' words itself, finished
+// 22 to 26 tiles per microsecond whatever the tile's size (hundreds of blocks read the words
+// that are being written), so a pass over 2^28 rows took 1.5 ms with 8192-row tiles and 3.0
+// with 4096-row tiles.
+constexpr int kScanners = kRadix / kWarp;
+constexpr int kScanTiles = 16;
+
+struct ScanShared {
+  uint32_t running[kWarp];  // rows of the digit in the chunks before `turn`
+  int64_t turn;             // chunk whose turn it is
+  int32_t gave_up;
+};
+
+template <int WARPS>
+__device__ void scan_tiles(const PassArgs& a, int scanner, int64_t tiles, ScanShared& sh) {
+  const int lane = threadIdx.x % kWarp, warp = threadIdx.x / kWarp;
+  if (threadIdx.x < kWarp) sh.running[threadIdx.x] = 0;
+  if (threadIdx.x == 0) {
+    sh.turn = 0;
+    sh.gave_up = 0;
   }
-  for (int i = tid; i < WARPS * kRadix; i += THREADS) (&whist[0][0])[i] = 0;
   __syncthreads();
-  const int64_t tile = tile_sh;
-  if (tile * TILE >= a.n) return;  // nothing issued on the barrier yet
-  const int64_t tile_row = tile * TILE;
-  const int valid = static_cast<int>((a.n - tile_row) < TILE ? (a.n - tile_row) : TILE);
-  const int bulk = valid & ~3;
-  // BlockLoad: keys and values of the tile, one bulk copy each.
-  if (tid == 0) {
-    const uint64_t pol = policy_evict_first();
-    const uint32_t bytes = static_cast<uint32_t>(bulk) * 4u;
-    mbar_arrive_expect_tx(&loaded, 2 * bytes);
-    if (bytes) {
-      bulk_load(skeys, a.keys_in + tile_row, bytes, &loaded, pol);
-      bulk_load(svals, a.vals_in + tile_row, bytes, &loaded, pol);
-    }
-  }
-  if (bulk < valid) {  // ragged end of the last tile
-    for (int i = bulk + tid; i < valid; i += THREADS) {
-      skeys[i] = a.keys_in[tile_row + i];
-      svals[i] = a.vals_in[tile_row + i];
-    }
-  }
-  const bool ok = mbar_wait_bounded(&loaded, 0, a.err);
-  if (__syncthreads_or(!ok)) {
-    if (tid == 0) mbar_wait_bounded(&loaded, 0, a.err);
-    return;
-  }
-
-  // Stable per-warp ranking, warp-striped: item i of lane l in warp w is tile position
-  // w*32*ITEMS + i*32 + l.  In round i the lanes holding the same digit are found with
-  // 8 ballots (one per digit bit); each gets (keys of that digit in earlier rounds) +
-  // (same-digit lanes below it).  Rows past the end take part in no group.
-  const uint32_t lt_mask = (1u << lane) - 1u;
-  int32_t key[ITEMS];
-  uint32_t rank[ITEMS];
-  // a full tile (all but possibly the last) ranks without per-item bounds predicates
-  auto rank_items = [&](auto full_tag) {
-    constexpr bool FULL = decltype(full_tag)::value;
+  volatile int64_t* turn = &sh.turn;
+  volatile int32_t* gave_up = &sh.gave_up;
+  volatile uint32_t* running = sh.running;
+  for (int64_t c = warp; c * kScanTiles < tiles; c += WARPS) {
+    const int64_t first = c * kScanTiles;
+    const int chunk = static_cast<int>(tiles - first < kScanTiles ? tiles - first : kScanTiles);
+    uint32_t* word = a.status + first * kRadix + scanner * kWarp + lane;  // the chunk's first tile
+    uint32_t w[kScanTiles];
 #pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-      const int pos = warp * WSEG + i * kWarp + lane;
-      const bool real = FULL || pos < valid;
-      key[i] = real ? skeys[pos] : 0;
-      const uint32_t d = real ? digit_of(key[i], PASS) : 0u;
-      uint32_t peers = FULL ? 0xFFFFFFFFu : __ballot_sync(0xFFFFFFFFu, real);
+    for (int r = 0; r < kScanTiles; ++r) w[r] = 0;
+    SpinGuard guard;
+    int handed = 0, there = 0;  // tiles whose prefixes are out; published tiles in front
+    while (handed < chunk) {
+      if (there < chunk) {
+#pragma unroll
+        for (int r = 0; r < kScanTiles; ++r)
+          if (r >= there && r < chunk && w[r] == 0u) w[r] = ld_relaxed_u32(word + r * kRadix);
+        there = 0;
+#pragma unroll
+        for (int r = 0; r < kScanTiles; ++r)
+          if (there == r && __all_sync(0xFFFFFFFFu, w[r] != 0u)) there = r + 1;
+      }
+      const bool mine = __shfl_sync(0xFFFFFFFFu, static_cast<int>(*turn == c), 0) != 0;
+      if (there == handed || !mine) {
+        if (!__all_sync(0xFFFFFFFFu, guard.go_on(&a.head->abort_word, a.wait_ns, a.err)) ||
+            __any_sync(0xFFFFFFFFu, *gave_up)) {
+          if (lane == 0) *gave_up = 1;
+          return;
+        }
+        continue;
+      }
+      __threadfence_block();
+      uint32_t run = running[lane];
+      if (there == chunk) {  // the turn goes on before the stores
+        uint32_t total = 0;
+#pragma unroll
+        for (int r = 0; r < kScanTiles; ++r) total += w[r] & kValueMask;
+        running[lane] = run + total;
+        __threadfence_block();
+        __syncwarp();
+        if (lane == 0) *turn = c + 1;
+      }
+#pragma unroll
+      for (int r = 0; r < kScanTiles; ++r) {
+        if (r >= handed && r < there) st_relaxed_u32(word + r * kRadix, kFlagInclusive | run);
+        run += w[r] & kValueMask;
+      }
+      handed = there;
+    }
+  }
+}
+
+// This tile's rows of one digit: counted in the tiles before it.  False when that never came.
+__device__ __forceinline__ bool prefix_of(const PassArgs& a, const uint32_t* word, uint32_t* excl) {
+  SpinGuard guard;
+  uint32_t w = ld_relaxed_u32(word);
+  while ((w >> 30) != 2u) {
+    if (!guard.go_on(&a.head->abort_word, a.wait_ns, a.err)) return false;
+    w = ld_relaxed_u32(word);
+  }
+  *excl = w & kValueMask;
+  return true;
+}
+
+// Ranks of a warp's rows among its rows of the same digit, in row order.  Round i holds item i
+// of every lane; a lane's rank is (rows of its digit in earlier rounds) + (lanes below it
+// with the same digit), rows past the end taking part in no group (FULL: there are none).
+// `table` has a (lanes of this round, rows so far) pair per digit, all zero at the start; the
+// second words are the warp's digit counts at the end.
+//
+// The lanes with the same digit are found in turn by eight ballots and by OR-ing the lane's bit
+// into the table: the ballots keep the ALU busy (68% of its peak when all rounds use them,
+// 123 instructions per row), the table the shared-memory pipe (83%, 78 instructions), and
+// alternating them uses both.  2^28 random pairs, whole sort: all ballots 4.91 ms, all table
+// 4.94, one round in two 4.74, one in four by either 4.79 and 4.89.  A shared-memory atomic
+// per row with a repair of the lanes that share a digit took 5.14 (its repair loop is serial).
+template <int ITEMS, bool FULL, typename Digit>
+__device__ __forceinline__ void rank_rows(const int32_t (&k)[ITEMS], int lim, const Digit& digit, uint2* table,
+                                          uint32_t (&r)[ITEMS]) {
+  const uint32_t lane_bit = 1u << (threadIdx.x % kWarp), below = lane_bit - 1u;
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) {
+    const bool real = FULL || i * kWarp < lim;
+    const uint32_t d = real ? digit(k[i]) : 0u;
+    const uint32_t entry = smem_u32(table + d);
+    uint32_t peers, before = 0;
+    if (i % 2 == 0) {
+      if (real) atomicOr(&table[d].x, lane_bit);
+      __syncwarp();
+      asm volatile("ld.volatile.shared.v2.u32 {%0, %1}, [%2];" : "=r"(peers), "=r"(before) : "r"(entry) : "memory");
+      __syncwarp();
+      if (real && (peers & below) == 0)
+        asm volatile("st.volatile.shared.v2.u32 [%0], {%1, %2};" ::"r"(entry), "r"(0u), "r"(before + __popc(peers))
+                     : "memory");
+    } else {
+      peers = FULL ? 0xFFFFFFFFu : __ballot_sync(0xFFFFFFFFu, real);
 #pragma unroll
       for (int b = 0; b < 8; ++b) {
         const uint32_t bit = (d >> b) & 1u;
         const uint32_t vote = __ballot_sync(0xFFFFFFFFu, bit);
         peers &= bit ? vote : ~vote;
       }
-      uint32_t before = 0;
-      if (real) before = whist[warp][d];
+      if (real) before = *reinterpret_cast<volatile uint32_t*>(&table[d].y);
       __syncwarp();
-      rank[i] = before + __popc(peers & lt_mask);
-      if (real && (peers & lt_mask) == 0) whist[warp][d] = before + __popc(peers);
-      __syncwarp();
+      if (real && (peers & below) == 0) *reinterpret_cast<volatile uint32_t*>(&table[d].y) = before + __popc(peers);
     }
-  };
+    r[i] = (d << 16) | (before + __popc(peers & below));
+    __syncwarp();
+  }
+}
+
+// One tile.
+template <int THREADS, int ITEMS, typename Digit>
+__device__ __forceinline__ void pass_tile(const PassArgs& a, const PassCols& cols, const Digit digit, int64_t tile,
+                                          int32_t* sk, int32_t* sv, PassShared<THREADS>& sh) {
+  constexpr int WARPS = THREADS / kWarp;
+  constexpr int TILE = THREADS * ITEMS;
+  static_assert(THREADS >= kRadix && TILE < 65536, "one thread per digit, 16-bit counters");
+  const int tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
+  const int64_t row0 = tile * TILE;
+  const int valid = static_cast<int>((a.n - row0) < TILE ? (a.n - row0) : TILE);
+  const int lim = valid - warp * (kWarp * ITEMS) - lane;  // item i of this thread exists while 32 i < lim
+  const int32_t* kin = cols.kin + row0 + warp * (kWarp * ITEMS) + lane;
+  const int32_t* vin = cols.vin + row0 + warp * (kWarp * ITEMS) + lane;
+  const uint64_t pol = policy_evict_first();
+  int32_t k[ITEMS];  // keys, then values
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) k[i] = i * kWarp < lim ? ld_stream(kin + i * kWarp, pol) : 0;
+  if (tid == 0 && valid >= 4)  // the values are read after the keys are placed: on their way to L2
+    bulk_prefetch_l2(cols.vin + row0, static_cast<uint32_t>(valid & ~3) * 4u);
+
+  // Stable per-warp ranking, warp-striped: item i of lane l in warp w is tile position
+  // w*32*ITEMS + i*32 + l, so the rows of round i come before those of round i + 1.
+  uint32_t r[ITEMS];  // digit << 16 | rank in the warp, then place in the tile
+  static_assert(WARPS * kRadix <= TILE, "the warps' tables fit the place of the sorted tile");
+  uint2* table = reinterpret_cast<uint2*>(sk) + warp * kRadix;
+  for (int i = lane; i < kRadix / 2; i += kWarp) reinterpret_cast<uint4*>(table)[i] = make_uint4(0, 0, 0, 0);
+  __syncwarp();
   if (valid == TILE)
-    rank_items(std::true_type{});
+    rank_rows<ITEMS, true>(k, lim, digit, table, r);
   else
-    rank_items(std::false_type{});
+    rank_rows<ITEMS, false>(k, lim, digit, table, r);
+  for (int i = lane; i < kRadix; i += kWarp) sh.whist[warp][i] = static_cast<uint16_t>(table[i].y);
   __syncthreads();
 
-  // Per digit: exclusive offsets of the warps and the tile's count.
-  unsigned int count = 0;
+  // Per digit: exclusive offsets of the warps, the tile's count (published for the later
+  // tiles) and its start in the tile.
+  uint32_t count = 0;
   if (tid < kRadix) {
 #pragma unroll
     for (int w = 0; w < WARPS; ++w) {
-      const unsigned int c = whist[w][tid];
-      whist[w][tid] = count;
+      const uint32_t c = sh.whist[w][tid];
+      sh.whist[w][tid] = static_cast<uint16_t>(count);
       count += c;
     }
-    // Tile-local exclusive scan across digits (threads 0..255 = 8 warps).
-    const unsigned int inc = static_cast<unsigned int>(warp_inclusive_scan(static_cast<int32_t>(count), lane));
-    if (lane == kWarp - 1) scan_tmp[warp] = inc;
-    tile_start[tid] = inc - count;
+    st_relaxed_u32(a.status + tile * kRadix + tid, kFlagAggregate | count);
+    const uint32_t inc = static_cast<uint32_t>(warp_inclusive_scan(static_cast<int32_t>(count), lane));
+    if (lane == kWarp - 1) sh.scan_tmp[warp] = inc;
+    sh.tile_start[tid] = inc - count;
   }
   __syncthreads();
+  if (tid < kRadix) {
+    uint32_t wbase = 0;
+    for (int w = 0; w < warp; ++w) wbase += sh.scan_tmp[w];
+    sh.tile_start[tid] += wbase;
+  }
+  __syncthreads();
+
+  // BlockShuffle: keys and values to their sorted positions of the tile
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i)
+    if (i * kWarp < lim) {
+      const uint32_t d = r[i] >> 16;
+      r[i] = sh.tile_start[d] + sh.whist[warp][d] + (r[i] & 0xFFFFu);
+      sk[r[i]] = k[i];
+    }
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i) k[i] = i * kWarp < lim ? ld_stream(vin + i * kWarp, pol) : 0;
+#pragma unroll
+  for (int i = 0; i < ITEMS; ++i)
+    if (i * kWarp < lim) sv[r[i]] = k[i];
+
+  // Global positions; the scanner has mostly answered by now.
   bool failed = false;
   if (tid < kRadix) {
-    unsigned int wbase = 0;
-    for (int w = 0; w < warp; ++w) wbase += scan_tmp[w];
-    tile_start[tid] += wbase;
-    // Decoupled look-back for digit tid over the earlier tiles.
-    uint32_t* st = a.status + tile * kRadix + tid;
-    unsigned int excl = 0;
-    if (tile == 0) {
-      st_relaxed_u32(st, kFlagInclusive | count);
-    } else {
-      st_relaxed_u32(st, kFlagAggregate | count);
-      int64_t p = tile - 1;
-      uint64_t t0 = 0;
-      bool timing = false;
-      while (p >= 0) {
-        const uint32_t w = ld_relaxed_u32(a.status + p * kRadix + tid);
-        const uint32_t flag = w >> 30;
-        if (flag == 0) {
-          if (!timing) {
-            t0 = global_timer_ns();
-            timing = true;
-          } else if (global_timer_ns() - t0 > a.wait_ns) {
-            set_error(a.err, CRYS_DEV_TIMEOUT);
-            st_relaxed_u32(a.abort_word, 1u);
-            failed = true;
-            break;
-          }
-          if (ld_relaxed_u32(a.abort_word)) {  // another block of this sort gave up
-            failed = true;
-            break;
-          }
-          continue;
-        }
-        timing = false;
-        excl += w & kValueMask;
-        if (flag == 2) break;
-        --p;
-      }
-      if (!failed) st_relaxed_u32(st, kFlagInclusive | (excl + count));
-    }
-    out_shift[tid] = static_cast<int32_t>(a.digit_base[tid] + excl - tile_start[tid]);
+    uint32_t excl = 0;
+    failed = !prefix_of(a, a.status + tile * kRadix + tid, &excl);
+    const uint32_t start = a.digit_base[tid] + excl;
     // the digit's run [start, start + count) of this tile must land inside the output
-    const int64_t start = static_cast<int64_t>(a.digit_base[tid]) + excl;
-    if (!failed && count && (start < 0 || start + count > a.n)) {
+    if (!failed && count && static_cast<int64_t>(start) + count > a.n) {
       set_error(a.err, CRYS_DEV_BOUNDS);
       failed = true;
     }
+    sh.out_shift[tid] = start - sh.tile_start[tid];
   }
   if (__syncthreads_or(failed)) return;
-
-  // BlockShuffle in place: keys to their sorted positions (every key of the tile is in
-  // some thread's registers), then values (read first, written after a barrier).
-#pragma unroll
-  for (int i = 0; i < ITEMS; ++i) {
-    const int pos = warp * WSEG + i * kWarp + lane;
-    if (pos < valid) {
-      const uint32_t d = digit_of(key[i], PASS);
-      rank[i] += tile_start[d] + whist[warp][d];
-      skeys[rank[i]] = key[i];
-    }
-  }
-#pragma unroll
-  for (int i = 0; i < ITEMS; ++i) {
-    const int pos = warp * WSEG + i * kWarp + lane;
-    key[i] = pos < valid ? svals[pos] : 0;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int i = 0; i < ITEMS; ++i) {
-    const int pos = warp * WSEG + i * kWarp + lane;
-    if (pos < valid) svals[rank[i]] = key[i];
-  }
-  __syncthreads();
   // BlockStore in sorted order: each digit run is written with consecutive addresses.
+#pragma unroll 4
   for (int i = tid; i < valid; i += THREADS) {
-    const int32_t k = skeys[i];
-    const int64_t g = static_cast<int64_t>(out_shift[digit_of(k, PASS)]) + i;  // checked per digit above
-    a.keys_out[g] = k;
-    a.vals_out[g] = svals[i];
+    const int32_t key = sk[i];
+    const uint32_t g = sh.out_shift[digit(key)] + static_cast<uint32_t>(i);  // checked per digit above
+    cols.kout[g] = key;
+    cols.vout[g] = sv[i];
   }
+}
+
+// Resident blocks per SM a tile shape's shared memory and 65536 registers allow.
+constexpr int pass_blocks(int threads, int items) {
+  const int smem = 227 * 1024 / (threads * items * 8 + threads * 16 + 4 * 1024);
+  const int regs = 65536 / (threads * (2 * items + 18));
+  return smem < regs ? smem : regs;
+}
+
+template <int THREADS, int ITEMS>
+__global__ void __launch_bounds__(THREADS, pass_blocks(THREADS, ITEMS)) sort_pass_kernel(const __grid_constant__ PassArgs a) {
+  constexpr int TILE = THREADS * ITEMS;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  int32_t* sk = reinterpret_cast<int32_t*>(smem_raw);  // the tile's keys in sorted order
+  int32_t* sv = sk + TILE;                             // and values
+  __shared__ PassShared<THREADS> sh;
+  const int tid = threadIdx.x;
+  const int passes = static_cast<int>(a.head->passes);
+  if (a.pass >= passes) return;
+  // the last pass writes to the output, the one before to the scratch, and so on
+  const bool to_out = (passes - 1 - a.pass) % 2 == 0;
+  PassCols cols;
+  cols.kin = a.pass == 0 ? a.keys_in : to_out ? a.keys_tmp : a.keys_out;
+  cols.vin = a.pass == 0 ? a.vals_in : to_out ? a.vals_tmp : a.vals_out;
+  cols.kout = to_out ? a.keys_out : a.keys_tmp;
+  cols.vout = to_out ? a.vals_out : a.vals_tmp;
+  const uint32_t shift = a.head->shift[a.pass], mask = a.head->mask[a.pass];
+  const bool buckets = a.head->buckets != 0;
+  const KeyRange range = a.head->range;
+  if (tid == 0)  // a sort whose earlier pass gave up does no further work (tile id past the end)
+    sh.tile = ld_relaxed_u32(&a.head->abort_word) ? 0xFFFFFFFFu : atomicAdd(&a.head->tile_counter[a.pass], 1u);
+  __syncthreads();
+  const uint32_t ticket = sh.tile;
+  if (ticket < static_cast<uint32_t>(kScanners)) {
+    __shared__ ScanShared scan;
+    scan_tiles<THREADS / kWarp>(a, static_cast<int>(ticket), (a.n + TILE - 1) / TILE, scan);
+    return;
+  }
+  const int64_t tile = static_cast<int64_t>(ticket) - kScanners + a.tile_base;
+  if (ticket == 0xFFFFFFFFu || tile * TILE >= a.n) return;
+  if (buckets)
+    pass_tile<THREADS, ITEMS>(a, cols, PassDigit<true>{range, shift, mask}, tile, sk, sv, sh);
+  else
+    pass_tile<THREADS, ITEMS>(a, cols, PassDigit<false>{KeyRange{}, shift, mask}, tile, sk, sv, sh);
 }
 
 struct Layout {
@@ -329,49 +617,79 @@ Layout layout(int64_t n) {
   return L;
 }
 
+// Where the bucket plan keeps its counts and first rows (2^bits words each), or NULL when
+// the scratch has no room for them: with up to 256 buckets in the starts of passes that the
+// plan does not run, otherwise behind the status words of the tile shape in use.
+uint32_t* bucket_words(char* temp, const Layout& L, int bits, int64_t tiles) {
+  if (bits <= 8) return reinterpret_cast<uint32_t*>(temp + L.base) + kRadix;
+  const size_t at = L.status + up256(static_cast<size_t>(tiles) * kRadix * 4);
+  const size_t need = (size_t{2} << bits) * 4;
+  return at + need <= L.total ? reinterpret_cast<uint32_t*>(temp + at) : nullptr;
+}
+
 template <int THREADS, int ITEMS>
-int run_passes(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out, int32_t* vals_out,
-               int64_t n, char* temp, const Layout& L, cudaStream_t s) {
+int run_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out, int32_t* vals_out, int64_t n, char* temp,
+             const Layout& L, cudaStream_t s) {
   constexpr int TILE = THREADS * ITEMS;
   const int64_t tiles = (n + TILE - 1) / TILE;
   const size_t smem = static_cast<size_t>(TILE) * 8;
-  using Kernel = void (*)(PassArgs);
-  const Kernel kernels[kPasses] = {sort_pass_kernel<THREADS, ITEMS, 0>, sort_pass_kernel<THREADS, ITEMS, 1>,
-                                   sort_pass_kernel<THREADS, ITEMS, 2>, sort_pass_kernel<THREADS, ITEMS, 3>};
-  for (int p = 0; p < kPasses; ++p)
-    if (!allow_smem(kernels[p], smem)) return CRYS_ECUDA;
-  int32_t* tk = reinterpret_cast<int32_t*>(temp + L.tmp_keys);
-  int32_t* tv = reinterpret_cast<int32_t*>(temp + L.tmp_vals);
-  const int32_t* src_k[kPasses] = {keys_in, tk, keys_out, tk};
-  const int32_t* src_v[kPasses] = {vals_in, tv, vals_out, tv};
-  int32_t* dst_k[kPasses] = {tk, keys_out, tk, keys_out};
-  int32_t* dst_v[kPasses] = {tv, vals_out, tv, vals_out};
+  auto kernel = sort_pass_kernel<THREADS, ITEMS>;
+  if (!allow_smem(kernel, smem)) return CRYS_ECUDA;
+  if (cudaMemsetAsync(temp + L.hist, 0, L.status - L.hist, s) != cudaSuccess) return CRYS_ECUDA;
+  SortHead* head = reinterpret_cast<SortHead*>(temp + L.counters);
+  uint32_t* base = reinterpret_cast<uint32_t*>(temp + L.base);
+  int32_t* err = device_error_word();
+  if (!err) return CRYS_ECUDA;
+  const int bits = n <= kMaxBucketRows ? range_bits(n, kLocalCap) : 0;
+  uint32_t* counts = bits ? bucket_words(temp, L, bits, tiles) : nullptr;
+  const int64_t buckets = int64_t{1} << bits;
+  if (counts) {
+    if (bits > 8 && cudaMemsetAsync(counts, 0, static_cast<size_t>(buckets) * 4, s) != cudaSuccess) return CRYS_ECUDA;
+    if (launch_key_range(keys_in, n, bits, &head->range, s) != CRYS_OK) return CRYS_ECUDA;
+    const size_t bins = static_cast<size_t>(buckets) * 2;
+    if (!allow_smem(count_buckets_kernel, size_t{2} << 16)) return CRYS_ECUDA;
+    // a block for every 16 rows per thread, at most one per SM
+    int64_t grid = (n + 16 * kCountThreads - 1) / (16 * kCountThreads);
+    if (grid > sm_count()) grid = sm_count();
+    count_buckets_kernel<<<static_cast<unsigned>(grid), kCountThreads, bins, s>>>(keys_in, n, bits, head, counts,
+                                                                                 counts + buckets, base);
+    note_launch();
+  }
+  int64_t hist_grid = (n + 16 * kHistThreads - 1) / (16 * kHistThreads);
+  if (hist_grid > sm_count() * 4) hist_grid = sm_count() * 4;
+  sort_hist_kernel<<<static_cast<unsigned>(hist_grid), kHistThreads, 0, s>>>(keys_in, n, reinterpret_cast<unsigned int*>(temp + L.hist),
+                                                                           head, base);
+  note_launch();
+  if (check_launch() != CRYS_OK) return CRYS_ECUDA;
   PassArgs a;
+  a.keys_in = keys_in;
+  a.vals_in = vals_in;
+  a.keys_tmp = reinterpret_cast<int32_t*>(temp + L.tmp_keys);
+  a.vals_tmp = reinterpret_cast<int32_t*>(temp + L.tmp_vals);
+  a.keys_out = keys_out;
+  a.vals_out = vals_out;
   a.n = n;
+  a.head = head;
   a.status = reinterpret_cast<uint32_t*>(temp + L.status);
-  a.abort_word = reinterpret_cast<unsigned int*>(temp + L.counters) + kPasses;
-  a.err = device_error_word();
-  if (!a.err) return CRYS_ECUDA;
+  a.err = err;
   uint32_t stall_base = 0;
   uint64_t stall_ns = kWaitBoundNs;
   take_stall(CRYS_OP_SORT, &stall_base, &stall_ns);  // a test's stall applies to the first pass
   for (int p = 0; p < kPasses; ++p) {
     a.tile_base = p == 0 ? stall_base : 0u;
     a.wait_ns = p == 0 ? stall_ns : kWaitBoundNs;
-    a.keys_in = src_k[p];
-    a.vals_in = src_v[p];
-    a.keys_out = dst_k[p];
-    a.vals_out = dst_v[p];
     a.pass = p;
-    a.digit_base = reinterpret_cast<unsigned int*>(temp + L.base) + p * kRadix;
-    a.tile_counter = reinterpret_cast<unsigned int*>(temp + L.counters) + p;
+    a.digit_base = base + p * kRadix;
     if (cudaMemsetAsync(a.status, 0, static_cast<size_t>(tiles) * kRadix * 4, s) != cudaSuccess)
       return CRYS_ECUDA;
-    kernels[p]<<<static_cast<unsigned int>(tiles), THREADS, smem, s>>>(a);
+    kernel<<<static_cast<unsigned int>(tiles + kScanners), THREADS, smem, s>>>(a);
     note_launch();
     if (check_launch() != CRYS_OK) return CRYS_ECUDA;
   }
-  return CRYS_OK;
+  if (!counts) return CRYS_OK;
+  LocalArgs l{keys_out, vals_out, keys_out, vals_out, counts + buckets, counts, static_cast<uint32_t>(n), err,
+              &head->buckets, &head->abort_word};
+  return launch_local_sort<false>(l, static_cast<unsigned>(buckets), s);
 }
 
 constexpr int kOp = CRYS_OP_SORT;
@@ -406,18 +724,20 @@ extern "C" int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t
     return CRYS_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   char* temp = static_cast<char*>(d_temp);
-  if (cudaMemsetAsync(temp + L.hist, 0, L.status - L.hist, s) != cudaSuccess) return CRYS_ECUDA;
-  const int hist_grid = sm_count() * 4;
-  sort_hist_kernel<<<hist_grid, kHistThreads, 0, s>>>(keys_in, n, reinterpret_cast<unsigned int*>(temp + L.hist));
-  note_launch();
-  sort_scan_kernel<<<1, kPasses * kWarp, 0, s>>>(reinterpret_cast<unsigned int*>(temp + L.hist),
-                                                 reinterpret_cast<unsigned int*>(temp + L.base));
-  note_launch();
-  if (check_launch() != CRYS_OK) return CRYS_ECUDA;
-  switch (tile_variant(kOp)) {
-    case 1: return run_passes<kTiles[kOp][1].threads, kTiles[kOp][1].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
-    case 2: return run_passes<kTiles[kOp][2].threads, kTiles[kOp][2].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
-    case 3: return run_passes<kTiles[kOp][3].threads, kTiles[kOp][3].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
-    default: return run_passes<kTiles[kOp][0].threads, kTiles[kOp][0].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
+  if (n <= kLocalCap) {  // one block sorts everything
+    uint32_t stall_base;
+    uint64_t stall_ns;
+    take_stall(CRYS_OP_SORT, &stall_base, &stall_ns);  // no tiles to stall: the request is used up
+    int32_t* err = device_error_word();
+    if (!err) return CRYS_ECUDA;
+    return launch_local_sort<false>(
+        LocalArgs{keys_in, vals_in, keys_out, vals_out, nullptr, nullptr, static_cast<uint32_t>(n), err}, 1, s);
+  }
+  // up to 2^20 rows (one pass by buckets) the smallest tile, so that more SMs have one
+  switch (n <= (1 << 20) ? kNumVariants[kOp] - 1 : tile_variant(kOp)) {
+    case 1: return run_sort<kTiles[kOp][1].threads, kTiles[kOp][1].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
+    case 2: return run_sort<kTiles[kOp][2].threads, kTiles[kOp][2].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
+    case 3: return run_sort<kTiles[kOp][3].threads, kTiles[kOp][3].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
+    default: return run_sort<kTiles[kOp][0].threads, kTiles[kOp][0].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
   }
 }
