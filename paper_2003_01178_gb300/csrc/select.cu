@@ -18,6 +18,8 @@
 // atomic (the paper's scheme); mode 1 (select_ordered_kernel) turns the tiles' counts into
 // positions in tile order (tile ids handed out in order by an atomic counter, so a tile
 // only waits on tiles that running blocks already hold) and the result is in input order.
+#include <cooperative_groups.h>
+
 #include <mutex>
 #include <type_traits>
 
@@ -483,6 +485,85 @@ __global__ void __launch_bounds__(THREADS + 2 * kWarp) select_ordered_kernel(Sel
   }
 }
 
+// ---------------------------------------------------------------- small columns
+//
+// Up to kSmallRows rows are selected by one cluster of 8 blocks, in input order: a block counts
+// its share of the rows, writes the count to every block's shared memory, and stores.
+// No scratch and no cleared counter, so the call is one launch; it is launches that bound
+// small calls (100,003 rows: 11.8 us per call with two clearings and the tiled kernel, 6.2 us
+// with this one).  The line is what 8 blocks hold in registers, 16 rows per thread.
+constexpr int kSmallBlocks = 8;
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallVec = 4;  // groups of 4 rows per thread
+constexpr int64_t kSmallRows = int64_t{kSmallBlocks} * kSmallThreads * kSmallVec * 4;
+
+__global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThreads)
+    select_small_kernel(const int32_t* __restrict__ x, int n, int32_t lo, uint32_t span, int32_t* __restrict__ out,
+                        long long* count) {
+  namespace cg = cooperative_groups;
+  constexpr int WARPS = kSmallThreads / kWarp;
+  __shared__ int32_t wtot[WARPS];
+  __shared__ int32_t totals_of[kSmallBlocks];  // every block's count, written by that block
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = static_cast<int>(cluster.block_rank());
+  const int tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
+  // this block's rows [first, last), 128 * vec consecutive ones per warp
+  const int share = ((n + kSmallBlocks - 1) / kSmallBlocks + 3) & ~3;
+  const int first = min(rank * share, n), last = min(first + share, n);
+  const int vec = (last - first + kSmallThreads * 4 - 1) / (kSmallThreads * 4);
+  const int row0 = first + warp * 128 * vec + lane * 4;
+  int32_t v[4 * kSmallVec];
+  uint32_t bits = 0;
+#pragma unroll
+  for (int j = 0; j < kSmallVec; ++j) {
+    const int r = row0 + j * 128;
+    if (j < vec && r + 4 <= last) {
+      const int4 q = *reinterpret_cast<const int4*>(x + r);  // first and r are multiples of 4
+      v[4 * j + 0] = q.x;
+      v[4 * j + 1] = q.y;
+      v[4 * j + 2] = q.z;
+      v[4 * j + 3] = q.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[4 * j + e] = j < vec && r + e < last ? x[r + e] : 0;
+    }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const bool hit = j < vec && r + e < last && static_cast<uint32_t>(v[4 * j + e]) - static_cast<uint32_t>(lo) <= span;
+      bits |= static_cast<uint32_t>(hit) << (4 * j + e);
+    }
+  }
+  // one warp scan of the lanes' counts of all groups (group j's in byte j), then the warps'
+  uint32_t packed = 0;
+#pragma unroll
+  for (int j = 0; j < kSmallVec; ++j) packed |= static_cast<uint32_t>(__popc((bits >> (4 * j)) & 0xFu)) << (8 * j);
+  const uint32_t incl = static_cast<uint32_t>(warp_inclusive_scan(static_cast<int32_t>(packed), lane));
+  const uint32_t excl = incl - packed, totals = __shfl_sync(0xFFFFFFFFu, incl, kWarp - 1);
+  if (lane == 0) wtot[warp] = static_cast<int32_t>((totals & 0xFFu) + ((totals >> 8) & 0xFFu) + ((totals >> 16) & 0xFFu) + (totals >> 24));
+  __syncthreads();
+  if (warp == 0) {
+    const int32_t t = wtot[lane];
+    const int32_t inc = warp_inclusive_scan(t, lane);
+    wtot[lane] = inc - t;
+    const int32_t total = __shfl_sync(0xFFFFFFFFu, inc, kWarp - 1);
+    if (lane < kSmallBlocks) *cluster.map_shared_rank(&totals_of[rank], lane) = total;
+  }
+  cluster.sync();  // the only one: after it a block reads its own copy of the counts
+  int base = 0;
+#pragma unroll
+  for (int b = 0; b < kSmallBlocks; ++b) base += b < rank ? totals_of[b] : 0;
+  if (rank == kSmallBlocks - 1 && tid == 0) *count = static_cast<long long>(base) + totals_of[rank];
+  int run = base + wtot[warp];
+#pragma unroll
+  for (int j = 0; j < kSmallVec; ++j) {
+    int pos = run + static_cast<int>((excl >> (8 * j)) & 0xFFu);
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if (bits & (1u << (4 * j + e))) out[pos++] = v[4 * j + e];
+    run += static_cast<int>((totals >> (8 * j)) & 0xFFu);
+  }
+}
+
 template <int THREADS, int ITEMS>
 int launch(SelectArgs a, bool ordered, cudaStream_t s) {
   constexpr int TILE = THREADS * ITEMS;
@@ -542,6 +623,16 @@ extern "C" int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, 
   if (n > 0 && !aligned16(x)) return CRYS_EINVAL;
   if (need && (reinterpret_cast<uintptr_t>(d_temp) & 255u)) return CRYS_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
+  uint32_t stall_base = 0;
+  uint64_t stall_ns = kWaitBoundNs;
+  const bool stalled = n > 0 && lo <= hi && order_preserving && take_stall(CRYS_OP_SELECT, &stall_base, &stall_ns);
+  if (n > 0 && n <= kSmallRows && lo <= hi && !stalled) {
+    select_small_kernel<<<kSmallBlocks, kSmallThreads, 0, s>>>(x, static_cast<int>(n), lo,
+                                                              static_cast<uint32_t>(hi) - static_cast<uint32_t>(lo), out,
+                                                              reinterpret_cast<long long*>(d_count));
+    note_launch();
+    return check_launch();
+  }
   if (cudaMemsetAsync(d_count, 0, sizeof(int64_t), s) != cudaSuccess) return CRYS_ECUDA;
   if (n == 0) return CRYS_OK;
   if (lo > hi) {  // empty range: nothing selected (d_count already zeroed)
@@ -570,7 +661,8 @@ extern "C" int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, 
     a.block_counter = static_cast<unsigned int*>(d_temp) + 1;
     a.abort_word = static_cast<unsigned int*>(d_temp) + 32;  // polled: not in the counters' line
     a.tile_state = reinterpret_cast<uint64_t*>(static_cast<char*>(d_temp) + 256);
-    take_stall(CRYS_OP_SELECT, &a.tile_base, &a.wait_ns);
+    a.tile_base = stall_base;
+    a.wait_ns = stall_ns;
     // only the words of the chosen shape's tiles are read
     const int64_t tile = static_cast<int64_t>(kTiles[kOp][variant].threads) * kTiles[kOp][variant].items;
     if (cudaMemsetAsync(d_temp, 0, 256 + static_cast<size_t>((n + tile - 1) / tile) * 8, s) != cudaSuccess)
