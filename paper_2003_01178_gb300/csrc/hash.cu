@@ -315,8 +315,7 @@ int crys_probe_aggregate(const int32_t* fk, const int32_t* payload, int64_t n, c
   using namespace crys;
   if (n < 0 || !valid_table(ht) || !d_sum) return CRYS_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(d_sum, 0, sizeof(int64_t), s) != cudaSuccess) return CRYS_ECUDA;
-  if (d_matches && cudaMemsetAsync(d_matches, 0, sizeof(int64_t), s) != cudaSuccess) return CRYS_ECUDA;
+  if (!clear_results(d_sum, d_matches, s)) return CRYS_ECUDA;
   if (n == 0) return CRYS_OK;
   if (!fk || !payload || !aligned16(fk) || !aligned16(payload)) return CRYS_EINVAL;
   ProbeArgs a;

@@ -27,6 +27,13 @@ bool take_stall(int op, uint32_t* first_tile, uint64_t* wait_ns);
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Clears a join's sum and, when asked for, its match count: one operation when they are neighbours.
+inline bool clear_results(int64_t* d_sum, int64_t* d_matches, cudaStream_t s) {
+  const bool together = d_matches == d_sum + 1;
+  if (cudaMemsetAsync(d_sum, 0, together ? 16 : 8, s) != cudaSuccess) return false;
+  return together || !d_matches || cudaMemsetAsync(d_matches, 0, 8, s) == cudaSuccess;
+}
+
 inline int check_launch() { return cudaGetLastError() == cudaSuccess ? CRYS_OK : CRYS_ECUDA; }
 
 inline uint32_t log2_pow2(uint64_t v) {
@@ -73,5 +80,11 @@ bool allow_smem(K kernel, size_t bytes) {
   if (bytes == 0) return true;
   return set_dynamic_smem(reinterpret_cast<const void*>(kernel), bytes);
 }
+
+// Sorts of one cooperative launch (smallsort.cu): whether n rows can take it, and the launch.
+// `head` is 256 bytes of scratch; the tmp columns hold n values each.
+bool small_sort_fits(int64_t n);
+int launch_small_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_tmp, int32_t* vals_tmp,
+                      int32_t* keys_out, int32_t* vals_out, int64_t n, void* head, cudaStream_t s);
 
 }  // namespace crys

@@ -244,24 +244,11 @@ static __device__ __noinline__ void local_sort_digits(const LocalArgs& a, LocalS
   }
 }
 
-// One block per bucket.  kLarge: buckets above kLocalCap are sorted through global memory
-// (needs kin != kout); without it they are reported (CRYS_DEV_BOUNDS) and left alone.
-template <bool kLarge>
-__global__ void __launch_bounds__(kLocalThreads, 3) local_sort_kernel(const __grid_constant__ LocalArgs a) {
-  extern __shared__ __align__(128) unsigned char local_smem[];
-  LocalShared& sh = *reinterpret_cast<LocalShared*>(local_smem);
+// Sorts rows [begin, begin + size) of one bucket, 1 <= size <= kLocalCap, by the whole block.
+// sh.loaded is an initialised barrier whose phases before `parity` are complete.
+__device__ __forceinline__ void local_sort_bucket(const LocalArgs& a, LocalShared& sh, uint32_t begin, uint32_t size,
+                                                  uint32_t parity) {
   const int tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
-  if ((a.go && *a.go == 0u) || (a.stop && *a.stop != 0u)) return;
-  const uint32_t begin = a.begin ? a.begin[blockIdx.x] : 0u;
-  const uint32_t size = a.begin ? a.count[blockIdx.x] : a.n;
-  if (size == 0) return;
-  if (size > static_cast<uint32_t>(kLocalCap)) {
-    if (kLarge)
-      local_sort_large(a, sh, begin, size);
-    else if (tid == 0)
-      set_error(a.err, CRYS_DEV_BOUNDS);
-    return;
-  }
   const int cnt = static_cast<int>(size);
   const int per = (cnt + kLocalThreads - 1) / kLocalThreads;  // rows per thread, warp-striped
   // the values travel to shared memory meanwhile: whole 16-byte groups by a bulk copy
@@ -269,8 +256,6 @@ __global__ void __launch_bounds__(kLocalThreads, 3) local_sort_kernel(const __gr
   const int skew = static_cast<int>((reinterpret_cast<uintptr_t>(vsrc) & 15u) / 4);
   const int bulk = (cnt + skew) & ~3;  // words copied, from the group that holds the first value
   if (tid == 0) {
-    mbar_init(&sh.loaded, 1);
-    fence_barrier_init();
     mbar_arrive_expect_tx(&sh.loaded, static_cast<uint32_t>(bulk) * 4u);
     if (bulk) bulk_load(sh.vals, vsrc - skew, static_cast<uint32_t>(bulk) * 4u, &sh.loaded, policy_evict_first());
   }
@@ -374,13 +359,37 @@ __global__ void __launch_bounds__(kLocalThreads, 3) local_sort_kernel(const __gr
   // the last 16-byte group of the values, when the copy did not cover it
   if (tid >= bulk - skew && tid < cnt && bulk <= skew) sh.vals[skew + tid] = vsrc[tid];
   if (bulk > skew && tid < cnt - (bulk - skew)) sh.vals[bulk + tid] = vsrc[bulk - skew + tid];
-  const bool ok = mbar_wait_bounded(&sh.loaded, 0, a.err);
+  const bool ok = mbar_wait_bounded(&sh.loaded, parity, a.err);
   if (__syncthreads_or(!ok)) return;
 #pragma unroll 4
   for (int q = tid; q < cnt; q += kLocalThreads) {
     a.kout[begin + q] = static_cast<int32_t>(sh.words[q]);
     a.vout[begin + q] = sh.vals[skew + sh.out.order[q]];
   }
+}
+
+// One block per bucket.  kLarge: buckets above kLocalCap are sorted through global memory
+// (needs kin != kout); without it they are reported (CRYS_DEV_BOUNDS) and left alone.
+template <bool kLarge>
+__global__ void __launch_bounds__(kLocalThreads, 3) local_sort_kernel(const __grid_constant__ LocalArgs a) {
+  extern __shared__ __align__(128) unsigned char local_smem[];
+  LocalShared& sh = *reinterpret_cast<LocalShared*>(local_smem);
+  if ((a.go && *a.go == 0u) || (a.stop && *a.stop != 0u)) return;
+  const uint32_t begin = a.begin ? a.begin[blockIdx.x] : 0u;
+  const uint32_t size = a.begin ? a.count[blockIdx.x] : a.n;
+  if (size == 0) return;
+  if (size > static_cast<uint32_t>(kLocalCap)) {
+    if (kLarge)
+      local_sort_large(a, sh, begin, size);
+    else if (threadIdx.x == 0)
+      set_error(a.err, CRYS_DEV_BOUNDS);
+    return;
+  }
+  if (threadIdx.x == 0) {
+    mbar_init(&sh.loaded, 1);
+    fence_barrier_init();
+  }
+  local_sort_bucket(a, sh, begin, size, 0);
 }
 
 // Sorts `buckets` buckets (one block each).

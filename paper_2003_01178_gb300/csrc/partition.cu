@@ -765,6 +765,9 @@ extern "C" int crys_sort_msb(const int32_t* keys_in, const int32_t* vals_in, int
   const uint32_t rows = static_cast<uint32_t>(n);
   if (bits == 0)  // one block sorts everything
     return launch_local_sort<false>(LocalArgs{keys_in, vals_in, keys_out, vals_out, nullptr, nullptr, rows, err}, 1, s);
+  // (its counts lie in the output's keys, read in 16-byte groups)
+  if (aligned16(keys_out) && small_sort_fits(n))
+    return launch_small_sort(keys_in, vals_in, tk, tv, keys_out, vals_out, n, range, s);
   if (launch_key_range(keys_in, n, bits, range, s) != CRYS_OK) return CRYS_ECUDA;
   // level A: the whole array by the leading 8 bits
   seg_init_kernel<<<1, 1, 0, s>>>(rows, kPartTile, A.seg_begin, A.seg_size, A.tile_start);
@@ -837,8 +840,7 @@ extern "C" int crys_join_partitioned(const int32_t* bkeys, const int32_t* bvals,
   }
   if (!d_sum) return CRYS_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(d_sum, 0, 8, s) != cudaSuccess) return CRYS_ECUDA;
-  if (d_matches && cudaMemsetAsync(d_matches, 0, 8, s) != cudaSuccess) return CRYS_ECUDA;
+  if (!clear_results(d_sum, d_matches, s)) return CRYS_ECUDA;
   if (nb == 0 || np == 0) return CRYS_OK;
   if (!d_temp || !temp_bytes) return CRYS_EINVAL;
   if (*temp_bytes < need) return CRYS_ENOMEM;

@@ -27,13 +27,13 @@
 #include "common.cuh"
 #include "keyrange.cuh"
 #include "localsort.cuh"
+#include "multisplit.cuh"
 #include "pipeline.cuh"
 #include "tiles.h"
 
 namespace crys {
 namespace {
 
-constexpr int kRadix = 256;
 constexpr int kPasses = 4;
 constexpr uint32_t kFlagAggregate = 1u << 30;
 constexpr uint32_t kFlagInclusive = 2u << 30;
@@ -395,53 +395,6 @@ __device__ __forceinline__ bool prefix_of(const PassArgs& a, const uint32_t* wor
   return true;
 }
 
-// Ranks of a warp's rows among its rows of the same digit, in row order.  Round i holds item i
-// of every lane; a lane's rank is (rows of its digit in earlier rounds) + (lanes below it
-// with the same digit), rows past the end taking part in no group (FULL: there are none).
-// `table` has a (lanes of this round, rows so far) pair per digit, all zero at the start; the
-// second words are the warp's digit counts at the end.
-//
-// The lanes with the same digit are found in turn by eight ballots and by OR-ing the lane's bit
-// into the table: the ballots keep the ALU busy (68% of its peak when all rounds use them,
-// 123 instructions per row), the table the shared-memory pipe (83%, 78 instructions), and
-// alternating them uses both.  2^28 random pairs, whole sort: all ballots 4.91 ms, all table
-// 4.94, one round in two 4.74, one in four by either 4.79 and 4.89.  A shared-memory atomic
-// per row with a repair of the lanes that share a digit took 5.14 (its repair loop is serial).
-template <int ITEMS, bool FULL, typename Digit>
-__device__ __forceinline__ void rank_rows(const int32_t (&k)[ITEMS], int lim, const Digit& digit, uint2* table,
-                                          uint32_t (&r)[ITEMS]) {
-  const uint32_t lane_bit = 1u << (threadIdx.x % kWarp), below = lane_bit - 1u;
-#pragma unroll
-  for (int i = 0; i < ITEMS; ++i) {
-    const bool real = FULL || i * kWarp < lim;
-    const uint32_t d = real ? digit(k[i]) : 0u;
-    const uint32_t entry = smem_u32(table + d);
-    uint32_t peers, before = 0;
-    if (i % 2 == 0) {
-      if (real) atomicOr(&table[d].x, lane_bit);
-      __syncwarp();
-      asm volatile("ld.volatile.shared.v2.u32 {%0, %1}, [%2];" : "=r"(peers), "=r"(before) : "r"(entry) : "memory");
-      __syncwarp();
-      if (real && (peers & below) == 0)
-        asm volatile("st.volatile.shared.v2.u32 [%0], {%1, %2};" ::"r"(entry), "r"(0u), "r"(before + __popc(peers))
-                     : "memory");
-    } else {
-      peers = FULL ? 0xFFFFFFFFu : __ballot_sync(0xFFFFFFFFu, real);
-#pragma unroll
-      for (int b = 0; b < 8; ++b) {
-        const uint32_t bit = (d >> b) & 1u;
-        const uint32_t vote = __ballot_sync(0xFFFFFFFFu, bit);
-        peers &= bit ? vote : ~vote;
-      }
-      if (real) before = *reinterpret_cast<volatile uint32_t*>(&table[d].y);
-      __syncwarp();
-      if (real && (peers & below) == 0) *reinterpret_cast<volatile uint32_t*>(&table[d].y) = before + __popc(peers);
-    }
-    r[i] = (d << 16) | (before + __popc(peers & below));
-    __syncwarp();
-  }
-}
-
 // One tile.
 template <int THREADS, int ITEMS, typename Digit>
 __device__ __forceinline__ void pass_tile(const PassArgs& a, const PassCols& cols, const Digit digit, int64_t tile,
@@ -629,7 +582,7 @@ uint32_t* bucket_words(char* temp, const Layout& L, int bits, int64_t tiles) {
 
 template <int THREADS, int ITEMS>
 int run_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out, int32_t* vals_out, int64_t n, char* temp,
-             const Layout& L, cudaStream_t s) {
+             const Layout& L, uint32_t stall_base, uint64_t stall_ns, cudaStream_t s) {
   constexpr int TILE = THREADS * ITEMS;
   const int64_t tiles = (n + TILE - 1) / TILE;
   const size_t smem = static_cast<size_t>(TILE) * 8;
@@ -672,9 +625,6 @@ int run_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out, 
   a.head = head;
   a.status = reinterpret_cast<uint32_t*>(temp + L.status);
   a.err = err;
-  uint32_t stall_base = 0;
-  uint64_t stall_ns = kWaitBoundNs;
-  take_stall(CRYS_OP_SORT, &stall_base, &stall_ns);  // a test's stall applies to the first pass
   for (int p = 0; p < kPasses; ++p) {
     a.tile_base = p == 0 ? stall_base : 0u;
     a.wait_ns = p == 0 ? stall_ns : kWaitBoundNs;
@@ -724,20 +674,24 @@ extern "C" int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t
     return CRYS_EINVAL;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   char* temp = static_cast<char*>(d_temp);
+  uint32_t stall_base = 0;
+  uint64_t stall_ns = kWaitBoundNs;
+  // a test's stall applies to the first pass: a stalled sort goes by passes (one block has no tiles)
+  const bool stalled = take_stall(CRYS_OP_SORT, &stall_base, &stall_ns);
   if (n <= kLocalCap) {  // one block sorts everything
-    uint32_t stall_base;
-    uint64_t stall_ns;
-    take_stall(CRYS_OP_SORT, &stall_base, &stall_ns);  // no tiles to stall: the request is used up
     int32_t* err = device_error_word();
     if (!err) return CRYS_ECUDA;
     return launch_local_sort<false>(
         LocalArgs{keys_in, vals_in, keys_out, vals_out, nullptr, nullptr, static_cast<uint32_t>(n), err}, 1, s);
   }
+  if (!stalled && small_sort_fits(n))
+    return launch_small_sort(keys_in, vals_in, reinterpret_cast<int32_t*>(temp + L.tmp_keys),
+                             reinterpret_cast<int32_t*>(temp + L.tmp_vals), keys_out, vals_out, n, temp + L.counters, s);
   // up to 2^20 rows (one pass by buckets) the smallest tile, so that more SMs have one
   switch (n <= (1 << 20) ? kNumVariants[kOp] - 1 : tile_variant(kOp)) {
-    case 1: return run_sort<kTiles[kOp][1].threads, kTiles[kOp][1].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
-    case 2: return run_sort<kTiles[kOp][2].threads, kTiles[kOp][2].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
-    case 3: return run_sort<kTiles[kOp][3].threads, kTiles[kOp][3].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
-    default: return run_sort<kTiles[kOp][0].threads, kTiles[kOp][0].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, s);
+    case 1: return run_sort<kTiles[kOp][1].threads, kTiles[kOp][1].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, stall_base, stall_ns, s);
+    case 2: return run_sort<kTiles[kOp][2].threads, kTiles[kOp][2].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, stall_base, stall_ns, s);
+    case 3: return run_sort<kTiles[kOp][3].threads, kTiles[kOp][3].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, stall_base, stall_ns, s);
+    default: return run_sort<kTiles[kOp][0].threads, kTiles[kOp][0].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, stall_base, stall_ns, s);
   }
 }
