@@ -153,8 +153,15 @@ def _ptr(t) -> int | None:
     return t.data_ptr()
 
 
+# The current stream's handle without building a Stream object for it (0.2 us against 2.9 us per
+# call on the GPU machine's host, of 6 to 20 us for a whole small operator call).
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None) -> int:
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(torch.cuda.current_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
@@ -223,8 +230,8 @@ def crys_hash_init(ht: crys_hash, stream=None) -> None:
 
 
 def crys_hash_build(keys, vals, n: int, filters: list, ht: crys_hash, stream=None) -> None:
-    arr = (crys_pred * max(1, len(filters)))(*[crys_pred(_ptr(c), lo, hi) for c, lo, hi in filters])
-    _check(lib().crys_hash_build(_ptr(keys), _ptr(vals), n, arr if filters else None, len(filters),
+    arr = (crys_pred * len(filters))(*[crys_pred(_ptr(c), lo, hi) for c, lo, hi in filters]) if filters else None
+    _check(lib().crys_hash_build(_ptr(keys), _ptr(vals), n, arr, len(filters),
                                  C.byref(ht), _stream(stream)), "crys_hash_build")
 
 
@@ -437,9 +444,10 @@ class HashTable:
 
 def probe_aggregate(fk: torch.Tensor, payload: torch.Tensor, ht: HashTable, stream=None):
     """(SUM(payload * value), matches) as int64 device tensors of one element."""
-    out = torch.zeros(2, dtype=torch.int64, device=fk.device)
-    crys_probe_aggregate(fk, payload, fk.numel(), ht.struct, out[0:1], out[1:2], stream)
-    return out[0:1], out[1:2]
+    # both are overwritten by the call; one allocation, so that one clearing covers both
+    total, matches = torch.empty(2, dtype=torch.int64, device=fk.device).split(1)
+    crys_probe_aggregate(fk, payload, fk.numel(), ht.struct, total, matches, stream)
+    return total, matches
 
 
 def sort(keys: torch.Tensor, vals: torch.Tensor, stream=None):
@@ -466,12 +474,11 @@ def sort_msb(keys: torch.Tensor, vals: torch.Tensor, stream=None):
 def join_partitioned(bkeys: torch.Tensor, bvals: torch.Tensor, fk: torch.Tensor, payload: torch.Tensor,
                      stream=None):
     """(SUM(payload * value), matches) of the radix-partitioned join, int64 device tensors."""
-    out = torch.zeros(2, dtype=torch.int64, device=fk.device)
+    total, matches = torch.empty(2, dtype=torch.int64, device=fk.device).split(1)
     tb = crys_join_partitioned(None, None, bkeys.numel(), None, None, fk.numel(), None, None, None, -1)
     temp = scratch(tb, fk.device)
-    crys_join_partitioned(bkeys, bvals, bkeys.numel(), fk, payload, fk.numel(), out[0:1], out[1:2], temp, tb,
-                          stream)
-    return out[0:1], out[1:2]
+    crys_join_partitioned(bkeys, bvals, bkeys.numel(), fk, payload, fk.numel(), total, matches, temp, tb, stream)
+    return total, matches
 
 
 def make_table(cols: list) -> crys_table:
