@@ -5,8 +5,8 @@
 // A cooperative launch of at most 304 blocks, each holding up to 4992 rows, with a grid
 // barrier between the steps:
 //  1. smallest and largest key;
-//  2. every block ranks its rows stably by the bucket of their key (256 buckets over the key
-//     range) and publishes its bucket counts;
+//  2. every block ranks its rows stably by the bucket of their key (up to 256 buckets over the
+//     key range) and publishes its bucket counts;
 //  3. every block sums the counts of the blocks before it and stores its rows, bucket by
 //     bucket, to the scratch columns;
 //  4. the blocks sort the buckets (localsort.cuh) into the output.  A key range of at most
@@ -44,7 +44,8 @@ struct SmallArgs {
   int32_t *keys_tmp, *vals_tmp;
   int32_t *keys_out, *vals_out;
   uint32_t n;
-  uint32_t share;  // rows per block
+  uint32_t share;    // rows per block
+  uint32_t buckets;  // at most kRadix
   SmallHead* head;
   int32_t* err;
 };
@@ -84,7 +85,7 @@ __device__ __forceinline__ bool grid_barrier(const SmallArgs& a, unsigned int k)
   return all;
 }
 
-// Bucket of a key: 256 over [lo, lo + span]; the key's offset itself for at most 256 values.
+// Bucket of a key: evenly over [lo, lo + span]; the key's offset itself for at most 256 values.
 struct BucketDigit {
   uint32_t lo, scale;
   __device__ __forceinline__ uint32_t operator()(int32_t k) const {
@@ -234,7 +235,7 @@ __global__ void __launch_bounds__(kThreads, 2) small_sort_kernel(const __grid_co
   const uint32_t span = hi - lo;
   const bool direct = span < kRadix;  // a bucket per value: nothing left to sort afterwards
   const BucketDigit bucket{lo ^ 0x80000000u,
-                           direct ? 0u : static_cast<uint32_t>((uint64_t{kRadix} << 32) / (static_cast<uint64_t>(span) + 1))};
+                           direct ? 0u : static_cast<uint32_t>((static_cast<uint64_t>(a.buckets) << 32) / (static_cast<uint64_t>(span) + 1))};
   // 2. counts; 3. stores.  The matrix lies in whichever of the two key columns is not written.
   uint32_t r[kItems];
   uint16_t* matrix = reinterpret_cast<uint16_t*>(direct ? a.keys_tmp : a.keys_out);
@@ -308,12 +309,18 @@ int launch_small_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* k
   int32_t* err = device_error_word();
   if (!err) return CRYS_ECUDA;
   if (cudaMemsetAsync(head, 0, sizeof(SmallHead), s) != cudaSuccess) return CRYS_ECUDA;
-  // a block per SM from 1024 rows per block, more blocks once they would hold too many
-  int64_t grid = (n + 1023) / 1024;
+  // A block per SM, fewer while their rows of counts would not fit the key column (2 bytes per
+  // count, 4 per row), more once they would hold too many rows.  As many buckets as blocks
+  // up to 2^18 rows, so that each block sorts one; then 256, so that a bucket fits a block.
+  // (With a block per 1024 rows and always 256 buckets, 5000 rows took 170 us, the blocks
+  // sorting 51 buckets each; 72 us by a dozen launches.)
+  int64_t grid = n / (kRadix / 2);
   if (grid > sm_count()) grid = sm_count();
   if (grid < (n + kRows - 1) / kRows) grid = (n + kRows - 1) / kRows;
+  uint32_t buckets = kRadix;
+  while (buckets > grid && n <= (1 << 18)) buckets /= 2;
   SmallArgs a{keys_in, vals_in, keys_tmp, vals_tmp, keys_out, vals_out, static_cast<uint32_t>(n),
-              static_cast<uint32_t>((n + grid - 1) / grid), static_cast<SmallHead*>(head), err};
+              static_cast<uint32_t>((n + grid - 1) / grid), buckets, static_cast<SmallHead*>(head), err};
   void* args[] = {&a};
   if (cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(small_sort_kernel), dim3(static_cast<unsigned>(grid)),
                                   dim3(kThreads), args, sizeof(SmallShared), s) != cudaSuccess)
