@@ -136,13 +136,13 @@ __device__ __forceinline__ void unpack4(int4 q, int32_t* dst) {
 // Probes one table for this thread's ITEMS rows: all first-slot reads are issued before
 // any is resolved.  (Continuations go item by item here: resolving them together, as the
 // probe kernel does, costs this kernel 20 more registers and half its resident blocks.)  Returns the bitmap of rows whose key was found; values in `value`.
-template <int ITEMS>
+template <int ITEMS, bool DIRECT = false>
 __device__ __forceinline__ uint32_t probe_items(const uint64_t* slots, const HashFn& hf,
                                                 const int32_t (&key)[ITEMS], uint32_t live,
                                                 int32_t (&value)[ITEMS], uint64_t pol) {
   uint32_t h[ITEMS];
   uint64_t slot[ITEMS];
-  if (hf.steps == 0u && hf.mult_hi == 1u && hf.mult_lo == 0u && hf.shift == 0u && hf.mask == 0xFFFFFFFFu) {
+  if (DIRECT || (hf.steps == 0u && hf.mult_hi == 1u && hf.mult_lo == 0u && hf.shift == 0u && hf.mask == 0xFFFFFFFFu)) {
     // direct table (uniform branch): a key below the capacity is in slot `key` or
     // absent, one read per row
     uint32_t found = 0;
@@ -157,17 +157,19 @@ __device__ __forceinline__ uint32_t probe_items(const uint64_t* slots, const Has
     }
     return found;
   }
+  uint32_t found = 0;
+  if constexpr (!DIRECT) {
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     h[i] = hash_slot(key[i], hf);
     slot[i] = ((live >> i) & 1u) && hash_may_hold(key[i], hf) ? ld_slot(slots + h[i], pol) : kEmptySlot;
   }
-  uint32_t found = 0;
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) {
     value[i] = 0;
     if (((live >> i) & 1u) && hash_resolve(slots, hf, h[i], slot[i], key[i], &value[i], pol))
       found |= 1u << i;
+  }
   }
   return found;
 }
@@ -414,7 +416,11 @@ __device__ __forceinline__ void load_tile_vectors(const DevQuery& q, const Cols&
 }
 
 // Evaluation of a tile whose leading column vectors are already in registers.
-template <int THREADS, int ITEMS, typename Cols>
+// DIRECT: every join is on a direct table.  Leaving the hashed probes out and not unrolling the
+// joins past the second keeps the kernel's code small: with both in, a warp waited for
+// instructions about as long as it issued them (three joins on direct tables, 60M rows: 0.462
+// ms, four joins 0.597; without 0.426 and 0.468).
+template <int THREADS, int ITEMS, bool DIRECT, typename Cols>
 __device__ __forceinline__ uint32_t eval_tile_vectors(const DevQuery& q, const Cols& cols,
                                                       const TileVectors<ITEMS>& tv, uint32_t alive,
                                                       int32_t (&gid)[ITEMS], int64_t (&val)[ITEMS],
@@ -448,17 +454,10 @@ __device__ __forceinline__ uint32_t eval_tile_vectors(const DevQuery& q, const C
   }
 #pragma unroll
   for (int i = 0; i < ITEMS; ++i) gid[i] = 0;
-#pragma unroll
-  for (int jn = 0; jn < CRYS_MAX_JOINS; ++jn) {
-    if (jn >= q.n_joins) break;
-    const DevJoin& J = q.joins[jn];
-    int32_t key[ITEMS], value[ITEMS];
-#pragma unroll
-    for (int j = 0; j < VEC; ++j) {
-      if (jn < KJ) unpack4(kv[jn < KJ ? jn : 0][j], key + 4 * j);
-      else unpack4(cols.load4(J.fk_col, (j * THREADS + tid) * 4), key + 4 * j);
-    }
-    alive &= probe_items<ITEMS>(J.slots, J.hash, key, alive, value, pol_table);
+  auto join = [&](const DevJoin& J, const int32_t (&key)[ITEMS]) {
+    int32_t value[ITEMS];
+    alive &= probe_items<ITEMS, DIRECT>(J.slots, J.hash, key, alive, value, pol_table);
+#pragma unroll 1
     for (int f = 0; f < J.n_fp; ++f) {
       const uint32_t sh = J.fp_shift[f], mk = J.fp_mask[f], span = J.fp_span[f];
       const int32_t lo = J.fp_lo[f];
@@ -481,6 +480,21 @@ __device__ __forceinline__ uint32_t eval_tile_vectors(const DevQuery& q, const C
         alive &= ~bad;
       }
     }
+  };
+#pragma unroll
+  for (int jn = 0; jn < KJ; ++jn) {
+    if (jn >= q.n_joins) break;
+    int32_t key[ITEMS];
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) unpack4(kv[jn][j], key + 4 * j);
+    join(q.joins[jn], key);
+  }
+#pragma unroll 1
+  for (int jn = KJ; jn < q.n_joins; ++jn) {  // not unrolled: the code of a tile should stay in the instruction cache
+    int32_t key[ITEMS];
+#pragma unroll
+    for (int j = 0; j < VEC; ++j) unpack4(cols.load4(q.joins[jn].fk_col, (j * THREADS + tid) * 4), key + 4 * j);
+    join(q.joins[jn], key);
   }
 #pragma unroll
   for (int j = 0; j < VEC; ++j) {
@@ -506,21 +520,21 @@ __device__ __forceinline__ uint32_t eval_tile_vectors(const DevQuery& q, const C
 // The same evaluation with every leading column load of the tile issued before any value
 // is used, so that one L2 round trip serves the tile instead of one per step; for tiles
 // of 4 or 8 rows per thread, where the loaded vectors fit in registers.
-template <int THREADS, int ITEMS>
+template <int THREADS, int ITEMS, bool DIRECT>
 __device__ __forceinline__ uint32_t eval_eager_preload(const DevQuery& q, const GlobalCols& cols, uint32_t alive,
                                                        int32_t (&gid)[ITEMS], int64_t (&val)[ITEMS],
                                                        int32_t* err, uint64_t pol_table) {
   TileVectors<ITEMS> r;
   load_tile_vectors<THREADS, ITEMS>(q, cols, r);
-  return eval_tile_vectors<THREADS, ITEMS>(q, cols, r, alive, gid, val, err, pol_table);
+  return eval_tile_vectors<THREADS, ITEMS, DIRECT>(q, cols, r, alive, gid, val, err, pol_table);
 }
 
-template <int THREADS, int ITEMS, bool PRELOAD>
+template <int THREADS, int ITEMS, bool PRELOAD, bool DIRECT>
 __device__ __forceinline__ uint32_t eval_eager(const DevQuery& q, const GlobalCols& cols, uint32_t alive,
                                                int32_t (&gid)[ITEMS], int64_t (&val)[ITEMS],
                                                int32_t* err, uint64_t pol_table) {
   if constexpr (PRELOAD && (ITEMS == 4 || ITEMS == 8)) {
-    return eval_eager_preload<THREADS, ITEMS>(q, cols, alive, gid, val, err, pol_table);
+    return eval_eager_preload<THREADS, ITEMS, DIRECT>(q, cols, alive, gid, val, err, pol_table);
   } else {
     return eval_eager_loop<THREADS, ITEMS>(q, cols, alive, gid, val, err, pol_table);
   }
@@ -620,9 +634,13 @@ __device__ __forceinline__ void prefetch_tile(const int32_t* const* cols, uint32
 }
 
 constexpr int kPrefetchTiles = 2;  // tiles of a block prefetched ahead of the one in work
+// The same for plan_kernel, whose dimension tables (37 MB for four) share L2 with the tiles in
+// flight: two tiles ahead of 456 blocks and 6 columns are 45 MB, and a three-join query over
+// 60M rows took 0.426 ms with them against 0.389 with one (one or two joins: no difference).
+constexpr int kPlanPrefetchTiles = 1;
 constexpr int kTagPrefetchTiles = 1;  // the same for the tagged scan, whose tiles stay in work longer
 
-template <int THREADS, int ITEMS, bool PRELOAD>
+template <int THREADS, int ITEMS, bool PRELOAD, bool DIRECT>
 __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ PlanArgs a) {
   constexpr int TILE = THREADS * ITEMS;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -643,7 +661,7 @@ __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ P
   const uint64_t pol = policy_evict_first();
   const uint64_t pol_table = policy_evict_last();
   if (threadIdx.x == 0)
-    for (int d = 0; d < kPrefetchTiles; ++d) {
+    for (int d = 0; d < kPlanPrefetchTiles; ++d) {
       const int64_t tt = blockIdx.x + static_cast<int64_t>(d) * gridDim.x;
       if (tt < ntiles) prefetch_tile(a.cols, a.col_mask, a.row_begin, tt, TILE, nrows);
     }
@@ -699,7 +717,7 @@ __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ P
     int64_t t = blockIdx.x;
     if (t < ntiles && !q.never) load(t, cur);
     for (; t < ntiles; t += gridDim.x) {
-      const int64_t ahead = t + static_cast<int64_t>(kPrefetchTiles) * gridDim.x;
+      const int64_t ahead = t + static_cast<int64_t>(kPlanPrefetchTiles) * gridDim.x;
       if (threadIdx.x == 0 && ahead < ntiles) prefetch_tile(a.cols, a.col_mask, a.row_begin, ahead, TILE, nrows);
       const GlobalCols cols = tile_cols(t);
       const int64_t tn = t + gridDim.x;
@@ -714,10 +732,10 @@ __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ P
       uint32_t alive = 0;
       if (!q.never) {
         if (cols.valid == TILE)
-          alive = eval_tile_vectors<THREADS, ITEMS>(q, full_cols(cols), cur, (1u << ITEMS) - 1u, gid, val, a.err,
+          alive = eval_tile_vectors<THREADS, ITEMS, DIRECT>(q, full_cols(cols), cur, (1u << ITEMS) - 1u, gid, val, a.err,
                                                     pol_table);
         else
-          alive = eval_tile_vectors<THREADS, ITEMS>(q, cols, cur, rows_present<THREADS, ITEMS>(cols.valid), gid, val,
+          alive = eval_tile_vectors<THREADS, ITEMS, DIRECT>(q, cols, cur, rows_present<THREADS, ITEMS>(cols.valid), gid, val,
                                                     a.err, pol_table);
       }
       accumulate(alive, gid, val);
@@ -727,7 +745,7 @@ __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ P
     uint32_t need_lines = 0, seen_lines = 0;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
       const bool sparse = a.late_mask && seen_lines >= 64u && 3u * need_lines < seen_lines;
-      const int64_t ahead = t + static_cast<int64_t>(kPrefetchTiles) * gridDim.x;
+      const int64_t ahead = t + static_cast<int64_t>(kPlanPrefetchTiles) * gridDim.x;
       if (threadIdx.x == 0 && ahead < ntiles)
         prefetch_tile(a.cols, sparse ? (a.col_mask & ~a.late_mask) : a.col_mask, a.row_begin, ahead, TILE, nrows);
       const GlobalCols cols = tile_cols(t);
@@ -737,7 +755,7 @@ __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ P
       if (!q.never) {
         const uint32_t present = rows_present<THREADS, ITEMS>(cols.valid);
         if (PRELOAD || !sparse)
-          alive = eval_eager<THREADS, ITEMS, PRELOAD>(q, cols, present, gid, val, a.err, pol_table);
+          alive = eval_eager<THREADS, ITEMS, PRELOAD, DIRECT>(q, cols, present, gid, val, a.err, pol_table);
         else
           alive = eval_eager_loop<THREADS, ITEMS, true>(q, cols, present, gid, val, a.err, pol_table);
       }
@@ -1807,11 +1825,16 @@ int launch_plan(PlanArgs& a, cudaStream_t s) {
   // table: 0.665 against 0.818 ms).  The step-by-step evaluation, with selective loads of
   // the late columns, remains for other tile shapes.
   const int64_t ntiles = (a.row_end - a.row_begin + TILE - 1) / TILE;
-  auto kl = plan_kernel<THREADS, ITEMS, false>;
+  auto kl = plan_kernel<THREADS, ITEMS, false, false>;
   if (!allow_smem(kl, smem)) return CRYS_ECUDA;
   int grid = persistent_grid(kl, THREADS, smem, ntiles);
   const bool preload = ITEMS == 4 || ITEMS == 8;
-  auto k = preload ? plan_kernel<THREADS, ITEMS, true> : kl;
+  auto is_direct = [](const HashFn& h) {
+    return h.steps == 0u && h.mult_hi == 1u && h.mult_lo == 0u && h.shift == 0u && h.mask == 0xFFFFFFFFu;
+  };
+  bool direct = true;
+  for (int j = 0; j < a.q.n_joins; ++j) direct = direct && is_direct(a.q.joins[j].hash);
+  auto k = !preload ? kl : direct ? plan_kernel<THREADS, ITEMS, true, true> : plan_kernel<THREADS, ITEMS, true, false>;
   if (preload) {
     if (!allow_smem(k, smem)) return CRYS_ECUDA;
     grid = persistent_grid(k, THREADS, smem, ntiles);
@@ -1819,8 +1842,7 @@ int launch_plan(PlanArgs& a, cudaStream_t s) {
   // a plan of the Q1 family: the kernel compiled for its shape
   const DevJoin& J0 = a.q.joins[0];
   const bool fixed = preload && a.q.acc_mode == kAccSingle && a.q.n_joins == 1 &&
-                     (a.q.n_preds == 1 || a.q.n_preds == 2) && J0.card <= 0 && J0.hash.steps == 0u &&
-                     J0.hash.mult_hi == 1u && J0.hash.mult_lo == 0u && J0.hash.shift == 0u && J0.hash.mask == 0xFFFFFFFFu &&
+                     (a.q.n_preds == 1 || a.q.n_preds == 2) && J0.card <= 0 && direct &&
                      (a.q.agg_op == CRYS_AGG_A_MUL_B || a.q.agg_op == CRYS_AGG_A);
   if (fixed) {
     const bool mul = a.q.agg_op == CRYS_AGG_A_MUL_B;
