@@ -612,6 +612,23 @@ __global__ void __launch_bounds__(256) zero_outputs_kernel(unsigned long long* s
   }
 }
 
+// Outputs of a batch's queries.
+struct ZeroBatch {
+  unsigned long long* sums[CRYS_MAX_PLANS];
+  unsigned long long* counts[CRYS_MAX_PLANS];
+  int64_t groups[CRYS_MAX_PLANS];
+};
+
+// Clears query blockIdx.y's sums and counts.
+__global__ void __launch_bounds__(256) zero_batch_kernel(const __grid_constant__ ZeroBatch z) {
+  const int q = blockIdx.y;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t g = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; g < z.groups[q]; g += stride) {
+    z.sums[q][g] = 0;
+    if (z.counts[q]) z.counts[q][g] = 0;
+  }
+}
+
 struct PlanArgs {
   const int32_t* cols[CRYS_MAX_COLS];
   int64_t row_begin, row_end;
@@ -1787,11 +1804,22 @@ int check_table(const crys_table* t) {
   return CRYS_OK;
 }
 
-int zero_outputs(const DevQuery& q, cudaStream_t s) {
-  if (cudaMemsetAsync(q.sums, 0, static_cast<size_t>(q.groups) * 8, s) != cudaSuccess) return CRYS_ECUDA;
-  if (q.counts && cudaMemsetAsync(q.counts, 0, static_cast<size_t>(q.groups) * 8, s) != cudaSuccess)
-    return CRYS_ECUDA;
-  return CRYS_OK;
+// Clears the outputs of a batch on the stream, in one launch (32 queries were 64 clearings of
+// about 2 us each, on the GPU as for the host).
+int zero_outputs(const DevQuery* q, int n_plans, cudaStream_t s) {
+  if (n_plans == 0) return CRYS_OK;
+  ZeroBatch z;
+  int64_t most = 1;
+  for (int i = 0; i < n_plans; ++i) {
+    z.sums[i] = q[i].sums;
+    z.counts[i] = q[i].counts;
+    z.groups[i] = q[i].groups;
+    if (q[i].groups > most) most = q[i].groups;
+  }
+  const int64_t zb = (most + 255) / 256, zcap = static_cast<int64_t>(sm_count()) * 4;
+  zero_batch_kernel<<<dim3(static_cast<unsigned>(zb < zcap ? zb : zcap), static_cast<unsigned>(n_plans)), 256, 0, s>>>(z);
+  note_launch();
+  return check_launch();
 }
 
 // Clears a query's outputs on the stream: the kernel the query kernel is launched behind
@@ -2487,7 +2515,7 @@ int crys_run_plans(const crys_table* fact, const crys_plan* plans, int32_t n_pla
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   int rc = a->err ? CRYS_OK : CRYS_ECUDA;
   if (rc == CRYS_OK && !(flags & CRYS_ACCUMULATE)) {
-    for (int qi = 0; qi < n_plans && rc == CRYS_OK; ++qi) rc = zero_outputs(a->q[qi], s);
+    rc = zero_outputs(a->q, n_plans, s);
   }
   if (rc == CRYS_OK && n_plans > 0 && row_end > row_begin) {
     constexpr int kOp = CRYS_OP_SHARED_SCAN;
@@ -2554,7 +2582,7 @@ int crys_run_plans_tagged(const crys_table* fact, const crys_plan* plans, int32_
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   if (rc == CRYS_OK && !S.err) rc = CRYS_ECUDA;
   if (rc == CRYS_OK && !(flags & CRYS_ACCUMULATE))
-    for (int qi = 0; qi < n_plans && rc == CRYS_OK; ++qi) rc = zero_outputs(q[qi], s);
+    rc = zero_outputs(q, n_plans, s);
   if (rc == CRYS_OK && n_plans > 0 && row_end > row_begin) {
     unsigned char* base = static_cast<unsigned char*>(scratch);
     constexpr int kOp = CRYS_OP_TAGGED_SCAN;
