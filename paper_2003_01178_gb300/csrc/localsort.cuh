@@ -12,7 +12,8 @@
 //
 // What bounds it: issue slots (about 60% busy) and about 39 shared-memory wavefronts per 32 rows
 // (atomics, the random bin and place accesses), against 24 at HBM speed.  65536 buckets of
-// 4096 rows: 1.78 ms; four stable 4-bit passes over (low bits, row) words took 3.94 ms.
+// 4096 rows: 1.59 ms (159 instructions per row; 1.79 with branches around every compare); four
+// stable 4-bit passes over (low bits, row) words took 3.94 ms.
 #pragma once
 
 #include "common.cuh"
@@ -283,14 +284,13 @@ __device__ __forceinline__ void local_sort_bucket(const LocalArgs& a, LocalShare
   const int bits = 32 - __clz(span);
   const int shift = bits > kLocalBinBits ? bits - kLocalBinBits : 0;
 #pragma unroll
-  for (int i = 0; i < kLocalItems; ++i)
-    if (i < per) {
-      v[i] -= static_cast<uint32_t>(lo);
-      if (i * kWarp < lim) {
-        const uint32_t bin = v[i] >> shift, half = 16u * (bin & 1u);
-        at[i] = (atomicAdd(&sh.bins[bin >> 1], 1u << half) >> half) & 0xFFFFu;  // rows of the bin before this one
-      }
-    }
+  for (int i = 0; i < kLocalItems; ++i) {
+    if (i >= per) break;
+    v[i] -= static_cast<uint32_t>(lo);
+    const uint32_t bin = v[i] >> shift, half = 16u * (bin & 1u);
+    at[i] = 0;
+    if (i * kWarp < lim) at[i] = (atomicAdd(&sh.bins[bin >> 1], 1u << half) >> half) & 0xFFFFu;  // rows of the bin before this one
+  }
   __syncthreads();
   // starts of the bins, 13 bits, with the bin's rows above them (7: seven or more): each
   // thread takes consecutive bins
@@ -322,37 +322,39 @@ __device__ __forceinline__ void local_sort_bucket(const LocalArgs& a, LocalShare
     const uint32_t low = (1u << shift) - 1u;
     auto word = [&](int i) { return ((v[i] & low) << kLocalBinBits) | static_cast<uint32_t>(p0 + i * kWarp); };
 #pragma unroll
-    for (int i = 0; i < kLocalItems; ++i)
-      if (i < per && i * kWarp < lim) {
-        const uint32_t entry = bins[v[i] >> shift];
-        sh.words[(entry & kStart) + at[i]] = word(i);
-        at[i] |= entry << 8;  // place in the bin (at most kLocalCrowded), start and rows of the bin
-      }
+    for (int i = 0; i < kLocalItems; ++i) {
+      if (i >= per) break;
+      const uint32_t entry = bins[v[i] >> shift];
+      if (i * kWarp < lim) sh.words[(entry & kStart) + at[i]] = word(i);
+      at[i] |= entry << 8;  // place in the bin (at most kLocalCrowded), start and rows of the bin
+    }
     __syncthreads();
-    // rank inside the bin: no other row in 61% of the cases, one in 30%, two in 8% (half a row
-    // per bin on average); the others are compared without a loop up to two
+    // Rank inside the bin: no other row in 61% of the cases, one in 30%, two in 8% (half a row
+    // per bin on average).  The next two rows of the bin, cyclically, are compared without a
+    // branch (in a smaller bin they are the row itself), more in a loop.
 #pragma unroll
-    for (int i = 0; i < kLocalItems; ++i)
-      if (i < per && i * kWarp < lim) {
-        const uint32_t r = at[i] & 255u, s = (at[i] >> 8) & kStart, rows = at[i] >> (8 + kLocalBinBits);
-        const uint32_t mine = word(i);
-        uint32_t less = 0;
-        if (rows > 1u) less += sh.words[s + (r + 1u < rows ? r + 1u : r + 1u - rows)] < mine;
-        if (rows > 2u) less += sh.words[s + (r + 2u < rows ? r + 2u : r + 2u - rows)] < mine;
-        if (rows > 3u) {
-          const uint32_t e = (rows < 7u ? s + rows : bins[(v[i] >> shift) + 1] & kStart);
-          less = 0;
-          for (uint32_t j = s; j < e; ++j) less += sh.words[j] < mine;
-        }
-        at[i] = s + less;
+    for (int i = 0; i < kLocalItems; ++i) {
+      if (i >= per) break;
+      const uint32_t r = at[i] & 255u, s = (at[i] >> 8) & kStart, rows = at[i] >> (8 + kLocalBinBits);
+      const uint32_t mine = word(i);
+      const uint32_t o1 = r + 1u == rows ? 0u : r + 1u, o2 = o1 + 1u == rows ? 0u : o1 + 1u;
+      uint32_t less = static_cast<uint32_t>(sh.words[s + o1] < mine) + static_cast<uint32_t>(sh.words[s + o2] < mine);
+      if (rows > 3u) {
+        const uint32_t e = (rows < 7u ? s + rows : bins[(v[i] >> shift) + 1] & kStart);
+        less = 0;
+        for (uint32_t j = s; j < e; ++j) less += sh.words[j] < mine;
       }
+      at[i] = s + less;
+    }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kLocalItems; ++i)
-      if (i < per && i * kWarp < lim) {
+    for (int i = 0; i < kLocalItems; ++i) {
+      if (i >= per) break;
+      if (i * kWarp < lim) {
         sh.words[at[i]] = v[i] + static_cast<uint32_t>(lo);
         sh.out.order[at[i]] = static_cast<uint16_t>(p0 + i * kWarp);
       }
+    }
   } else {
     local_sort_digits(a, sh, begin, cnt, per, lo, bits);
   }
