@@ -660,6 +660,7 @@ constexpr int kTagPrefetchTiles = 1;  // the same for the tagged scan, whose til
 template <int THREADS, int ITEMS, bool PRELOAD, bool DIRECT>
 __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ PlanArgs a) {
   constexpr int TILE = THREADS * ITEMS;
+  constexpr int kAhead = DIRECT ? kPlanPrefetchTiles : kPrefetchTiles;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   __shared__ uint64_t red[THREADS / kWarp];
   const DevQuery& q = a.q;
@@ -678,7 +679,7 @@ __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ P
   const uint64_t pol = policy_evict_first();
   const uint64_t pol_table = policy_evict_last();
   if (threadIdx.x == 0)
-    for (int d = 0; d < kPlanPrefetchTiles; ++d) {
+    for (int d = 0; d < kAhead; ++d) {
       const int64_t tt = blockIdx.x + static_cast<int64_t>(d) * gridDim.x;
       if (tt < ntiles) prefetch_tile(a.cols, a.col_mask, a.row_begin, tt, TILE, nrows);
     }
@@ -734,7 +735,7 @@ __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ P
     int64_t t = blockIdx.x;
     if (t < ntiles && !q.never) load(t, cur);
     for (; t < ntiles; t += gridDim.x) {
-      const int64_t ahead = t + static_cast<int64_t>(kPlanPrefetchTiles) * gridDim.x;
+      const int64_t ahead = t + static_cast<int64_t>(kAhead) * gridDim.x;
       if (threadIdx.x == 0 && ahead < ntiles) prefetch_tile(a.cols, a.col_mask, a.row_begin, ahead, TILE, nrows);
       const GlobalCols cols = tile_cols(t);
       const int64_t tn = t + gridDim.x;
@@ -762,7 +763,7 @@ __global__ void __launch_bounds__(THREADS) plan_kernel(const __grid_constant__ P
     uint32_t need_lines = 0, seen_lines = 0;
     for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
       const bool sparse = a.late_mask && seen_lines >= 64u && 3u * need_lines < seen_lines;
-      const int64_t ahead = t + static_cast<int64_t>(kPlanPrefetchTiles) * gridDim.x;
+      const int64_t ahead = t + static_cast<int64_t>(kAhead) * gridDim.x;
       if (threadIdx.x == 0 && ahead < ntiles)
         prefetch_tile(a.cols, sparse ? (a.col_mask & ~a.late_mask) : a.col_mask, a.row_begin, ahead, TILE, nrows);
       const GlobalCols cols = tile_cols(t);
