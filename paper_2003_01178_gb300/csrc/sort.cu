@@ -7,7 +7,8 @@
 //    key's place between the smallest and largest key of a sample (keyrange.cuh), so narrow
 //    ranges fill the buckets too.  One kernel reads the keys and counts all buckets, which
 //    gives the passes' bucket starts and shows whether any bucket is too large for a block.
-//  * digits: when one is (heavily repeated or clustered keys), or there are too many rows, the
+//  * digits: when one is (heavily repeated or clustered keys), when a sample of the keys differs
+//    in at most three bytes (keyrange.cuh), or when there are too many rows, the
 //    least-significant-digit sort: 8-bit digits, a stable pass per digit from the low one to
 //    the high one.  Digits that have one value in all keys are skipped.
 //
@@ -52,7 +53,7 @@ struct SortHead {
   unsigned int abort_word;   // set by the first block of this sort that gives up
   unsigned int counted;      // blocks of the counting kernels that have finished
   unsigned int digits_counted;
-  unsigned int crowded;      // a bucket is too large for a block
+  unsigned int crowded;      // a bucket is too large for a block, or the keys differ in few bytes
   uint32_t buckets;          // 1: sorted by buckets, 0: by digits
   uint32_t passes;           // passes that do work; pass j writes to the output when an even number follows
   KeyRange range;
@@ -106,6 +107,7 @@ __global__ void __launch_bounds__(kCountThreads, 1) count_buckets_kernel(const i
   __shared__ unsigned int ticket;
   const int tid = threadIdx.x, lane = tid % kWarp, warp = tid / kWarp;
   const int words = 1 << (bits - 1);
+  if (__syncthreads_or(head->crowded != 0u)) return;  // decided already (head->buckets stays 0)
   for (int i = tid; i < words; i += kCountThreads) bins[i] = 0;
   const KeyRange range = head->range;
   const uint64_t pol = policy_evict_first();
@@ -598,7 +600,7 @@ int run_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out, 
   const int64_t buckets = int64_t{1} << bits;
   if (counts) {
     if (bits > 8 && cudaMemsetAsync(counts, 0, static_cast<size_t>(buckets) * 4, s) != cudaSuccess) return CRYS_ECUDA;
-    if (launch_key_range(keys_in, n, bits, &head->range, s) != CRYS_OK) return CRYS_ECUDA;
+    if (launch_key_range(keys_in, n, bits, &head->range, &head->crowded, s) != CRYS_OK) return CRYS_ECUDA;
     const size_t bins = static_cast<size_t>(buckets) * 2;
     if (!allow_smem(count_buckets_kernel, size_t{2} << 16)) return CRYS_ECUDA;
     // a block for every 16 rows per thread, at most one per SM

@@ -88,3 +88,22 @@ def test_msb_sort_unaligned_columns(crys):
             ko, vo = crys.sort_msb(k, v)
             rk, order = torch.sort(k, stable=True)
             assert torch.equal(ko, rk) and torch.equal(k[(vo - (3 - off)).long()], rk)
+
+
+# keys that differ in few bytes (the stable sort goes by digits), and the same with rare keys
+# outside the sample that differ in the others
+@pytest.mark.parametrize("rare", [False, True])
+@pytest.mark.parametrize("mask", [0x000000FF, 0x00FF00FF, 0x7FFF00FF, -0x10000, -0xFF0001, 0x00FFFFFF])
+@pytest.mark.parametrize("n", [(1 << 20) + 1, 3_000_017])
+def test_sorts_of_keys_with_few_bytes(crys, n, mask, rare):
+    keys = _keys("bits", n) & mask
+    if rare:
+        keys[n // 7 + 5] = -2
+        keys[n // 5 + 77] = I32_MAX - 255
+    vals = torch.arange(n, dtype=torch.int32, device="cuda")
+    rk, order = torch.sort(keys, stable=True)
+    ko, vo = crys.sort(keys, vals)
+    assert torch.equal(ko, rk) and torch.equal(vo, order.to(torch.int32))
+    ko, vo = crys.sort_msb(keys, vals)
+    assert torch.equal(ko, rk) and torch.equal(keys[vo.long()], rk)
+    assert torch.equal(vo.sort().values, vals)
