@@ -491,11 +491,14 @@ __global__ void __launch_bounds__(THREADS + 2 * kWarp) select_ordered_kernel(Sel
 // its share of the rows, writes the count to every block's shared memory, and stores.
 // No scratch and no cleared counter, so the call is one launch; it is launches that bound
 // small calls (100,003 rows: 11.8 us per call with two clearings and the tiled kernel, 6.2 us
-// with this one).  The line is what 8 blocks hold in registers, 16 rows per thread.
+// with this one).  The line is what 8 blocks hold in registers, 16 rows per thread; without an
+// order half of that, for the tiled kernel needs one clearing less there (all of 65536 rows 6.3
+// against 6.8 us, all of 131072 rows 8.2 against 6.5).
 constexpr int kSmallBlocks = 8;
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallVec = 4;  // groups of 4 rows per thread
 constexpr int64_t kSmallRows = int64_t{kSmallBlocks} * kSmallThreads * kSmallVec * 4;
+constexpr int64_t kSmallRowsAnyOrder = kSmallRows / 2;
 
 __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThreads)
     select_small_kernel(const int32_t* __restrict__ x, int n, int32_t lo, uint32_t span, int32_t* __restrict__ out,
@@ -626,7 +629,7 @@ extern "C" int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, 
   uint32_t stall_base = 0;
   uint64_t stall_ns = kWaitBoundNs;
   const bool stalled = n > 0 && lo <= hi && order_preserving && take_stall(CRYS_OP_SELECT, &stall_base, &stall_ns);
-  if (n > 0 && n <= kSmallRows && lo <= hi && !stalled) {
+  if (n > 0 && n <= (order_preserving ? kSmallRows : kSmallRowsAnyOrder) && lo <= hi && !stalled) {
     select_small_kernel<<<kSmallBlocks, kSmallThreads, 0, s>>>(x, static_cast<int>(n), lo,
                                                               static_cast<uint32_t>(hi) - static_cast<uint32_t>(lo), out,
                                                               reinterpret_cast<long long*>(d_count));

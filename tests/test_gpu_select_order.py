@@ -38,17 +38,18 @@ def test_ordered_select_at_chunk_edges(crys, variant, tiles):
     crys.crys_set_tile(crys.OP_SELECT, 0)
 
 
-@pytest.mark.parametrize("n", [1, 2, 5, 31, 33, 4095, 4097, 32_767, 32_769, 100_003, 131_071, 131_072, 131_073])
+@pytest.mark.parametrize("n", [1, 2, 5, 31, 33, 4095, 4097, 32_767, 32_769, 65_535, 65_536, 65_537, 100_003, 131_071, 131_072, 131_073])
 @pytest.mark.parametrize("ordered", [False, True])
 def test_select_of_one_cluster(crys, n, ordered):
-    # up to 131072 rows one cluster of 8 blocks selects, in input order in either mode
+    # one cluster of 8 blocks selects up to 131072 rows, 65536 without an order to keep (and keeps
+    # it all the same)
     g = torch.Generator(device="cuda")
     g.manual_seed(n)
     x = torch.randint(I32_MIN, I32_MAX, (n,), dtype=torch.int64, device="cuda", generator=g).to(torch.int32)
     for lo, hi in [(I32_MIN, I32_MAX), (0, I32_MAX), (-(1 << 28), 1 << 20), (int(x[n // 2]), int(x[n // 2])), (1, 0)]:
         got = crys.select(x, lo, hi, order_preserving=ordered)
         ref = x[(x >= lo) & (x <= hi)]
-        if n <= 131_072 or ordered:
+        if n <= 65_536 or ordered:
             assert torch.equal(got, ref), (lo, hi)
         else:
             assert torch.equal(got.sort().values, ref.sort().values), (lo, hi)
