@@ -1836,6 +1836,27 @@ int launch_zero_outputs(const DevQuery& q, cudaStream_t s) {
 // Per-block accumulators are 32-bit counts: a block must see fewer than 2^32 rows.
 bool counts_fit(int64_t rows, int grid) { return (rows / (grid > 0 ? grid : 1)) + (1 << 16) < (1ll << 32); }
 
+// Every join is on a direct table.
+bool all_direct(const DevQuery& q) {
+  for (int j = 0; j < q.n_joins; ++j) {
+    const HashFn& h = q.joins[j].hash;
+    if (h.steps != 0u || h.mult_hi != 1u || h.mult_lo != 0u || h.shift != 0u || h.mask != 0xFFFFFFFFu) return false;
+  }
+  return true;
+}
+
+// A plan of the Q1 family: one or two predicates, one join on a direct table without a group
+// code, one sum.
+bool of_fixed_shape(const DevQuery& q) {
+  return q.groups == 1 && q.n_joins == 1 && (q.n_preds == 1 || q.n_preds == 2) && q.joins[0].card <= 0 && all_direct(q) &&
+         (q.agg_op == CRYS_AGG_A_MUL_B || q.agg_op == CRYS_AGG_A);
+}
+
+// Rows up to which the default shape takes its smaller tiles for plans of the Q1 family: the
+// last tiles of so few rows leave much of the chip idle (12,000,001 rows 31.4 us with 256 x 8,
+// 32.9 with 512 x 8; 17,000,003 rows 43.2 and 43.5; 2^25 rows 80.4 and 79.5).
+constexpr int64_t kSmallTileRows = int64_t{3} << 23;
+
 template <int THREADS, int ITEMS>
 int launch_plan(PlanArgs& a, cudaStream_t s) {
   constexpr int TILE = THREADS * ITEMS;
@@ -1858,22 +1879,14 @@ int launch_plan(PlanArgs& a, cudaStream_t s) {
   if (!allow_smem(kl, smem)) return CRYS_ECUDA;
   int grid = persistent_grid(kl, THREADS, smem, ntiles);
   const bool preload = ITEMS == 4 || ITEMS == 8;
-  auto is_direct = [](const HashFn& h) {
-    return h.steps == 0u && h.mult_hi == 1u && h.mult_lo == 0u && h.shift == 0u && h.mask == 0xFFFFFFFFu;
-  };
-  bool direct = true;
-  for (int j = 0; j < a.q.n_joins; ++j) direct = direct && is_direct(a.q.joins[j].hash);
+  const bool direct = all_direct(a.q);
   auto k = !preload ? kl : direct ? plan_kernel<THREADS, ITEMS, true, true> : plan_kernel<THREADS, ITEMS, true, false>;
   if (preload) {
     if (!allow_smem(k, smem)) return CRYS_ECUDA;
     grid = persistent_grid(k, THREADS, smem, ntiles);
   }
   // a plan of the Q1 family: the kernel compiled for its shape
-  const DevJoin& J0 = a.q.joins[0];
-  const bool fixed = preload && a.q.acc_mode == kAccSingle && a.q.n_joins == 1 &&
-                     (a.q.n_preds == 1 || a.q.n_preds == 2) && J0.card <= 0 && direct &&
-                     (a.q.agg_op == CRYS_AGG_A_MUL_B || a.q.agg_op == CRYS_AGG_A);
-  if (fixed) {
+  if (preload && of_fixed_shape(a.q)) {
     const bool mul = a.q.agg_op == CRYS_AGG_A_MUL_B;
     if (a.q.n_preds == 2)
       k = mul ? plan_fixed_kernel<THREADS, ITEMS, 2, CRYS_AGG_A_MUL_B> : plan_fixed_kernel<THREADS, ITEMS, 2, CRYS_AGG_A>;
@@ -2443,7 +2456,11 @@ int crys_run_plan(const crys_table* fact, const crys_plan* plan, crys_stream str
     case 1: return launch_plan<kTiles[kOp][1].threads, kTiles[kOp][1].items>(a, s);
     case 2: return launch_plan<kTiles[kOp][2].threads, kTiles[kOp][2].items>(a, s);
     case 3: return launch_plan<kTiles[kOp][3].threads, kTiles[kOp][3].items>(a, s);
-    default: return launch_plan<kTiles[kOp][0].threads, kTiles[kOp][0].items>(a, s);
+    default:
+      static_assert(kTiles[kOp][1].threads == 256 && kTiles[kOp][1].items == 8, "the default shape's smaller tiles");
+      if (fact->n_rows <= kSmallTileRows && of_fixed_shape(a.q))
+        return launch_plan<kTiles[kOp][1].threads, kTiles[kOp][1].items>(a, s);
+      return launch_plan<kTiles[kOp][0].threads, kTiles[kOp][0].items>(a, s);
   }
 }
 
