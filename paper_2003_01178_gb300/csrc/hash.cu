@@ -333,7 +333,16 @@ int crys_probe_aggregate(const int32_t* fk, const int32_t* payload, int64_t n, c
     case 1: return launch_probe<kTiles[kOp][1].threads, kTiles[kOp][1].items>(a, s);
     case 2: return launch_probe<kTiles[kOp][2].threads, kTiles[kOp][2].items>(a, s);
     case 3: return launch_probe<kTiles[kOp][3].threads, kTiles[kOp][3].items>(a, s);
-    default: return launch_probe<kTiles[kOp][0].threads, kTiles[kOp][0].items>(a, s);
+    default:
+      // Tables too large to copy that L1 still holds, all or a good part of: with many probes the
+      // larger tiles, whose fewer blocks leave L1 more room, are ahead or equal (2^28 probes of
+      // tables of 64, 128, 256 and 512 KB: 0.484, 0.552, 0.992 and 0.956 ms with 256 x 16, 0.496,
+      // 0.553, 1.021 and 0.962 with 256 x 8; of 1 MB 0.985 and 0.913; 2^24 probes of 64 and 512
+      // KB 42.0 and 68.9 us against 39.3 and 66.2).
+      static_assert(kTiles[kOp][1].threads == 256 && kTiles[kOp][1].items == 16, "the larger tiles");
+      if (a.table_slots == 0 && ht->capacity * 8 <= 16 * kSmemTableBytes && n >= (1 << 25))
+        return launch_probe<kTiles[kOp][1].threads, kTiles[kOp][1].items>(a, s);
+      return launch_probe<kTiles[kOp][0].threads, kTiles[kOp][0].items>(a, s);
   }
 }
 
