@@ -488,7 +488,8 @@ __global__ void __launch_bounds__(THREADS + 2 * kWarp) select_ordered_kernel(Sel
 // ---------------------------------------------------------------- small columns
 //
 // Up to kSmallRows rows are selected by one cluster of 8 blocks, in input order: a block counts
-// its share of the rows, writes the count to every block's shared memory, and stores.
+// its share of the rows, writes the count to every block's shared memory, and stores.  The
+// wait that shows that the other blocks run lies behind the loads and the block's own count.
 // No scratch and no cleared counter, so the call is one launch; it is launches that bound
 // small calls (100,003 rows: 11.8 us per call with two clearings and the tiled kernel, 6.2 us
 // with this one).  The line is what 8 blocks hold in registers, 16 rows per thread; without an
@@ -502,8 +503,9 @@ constexpr int64_t kSmallRowsAnyOrder = kSmallRows / 2;
 
 __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThreads)
     select_small_kernel(const int32_t* __restrict__ x, int n, int32_t lo, uint32_t span, int32_t* __restrict__ out,
-                        long long* count) {
+                        long long* count, int32_t* err) {
   namespace cg = cooperative_groups;
+  cluster_arrive_relaxed();  // this block runs; waited for before the first store to another block
   constexpr int WARPS = kSmallThreads / kWarp;
   __shared__ int32_t wtot[WARPS];
   __shared__ int32_t totals_of[kSmallBlocks];  // every block's count, written by that block
@@ -544,6 +546,7 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
   const uint32_t excl = incl - packed, totals = __shfl_sync(0xFFFFFFFFu, incl, kWarp - 1);
   if (lane == 0) wtot[warp] = static_cast<int32_t>((totals & 0xFFu) + ((totals >> 8) & 0xFFu) + ((totals >> 16) & 0xFFu) + (totals >> 24));
   __syncthreads();
+  cluster_wait();  // every block runs: their shared memory may be written
   if (warp == 0) {
     const int32_t t = wtot[lane];
     const int32_t inc = warp_inclusive_scan(t, lane);
@@ -551,10 +554,14 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
     const int32_t total = __shfl_sync(0xFFFFFFFFu, inc, kWarp - 1);
     if (lane < kSmallBlocks) *cluster.map_shared_rank(&totals_of[rank], lane) = total;
   }
-  cluster.sync();  // the only one: after it a block reads its own copy of the counts
+  cluster.sync();  // the counts are there: a block reads its own copy of them
   int base = 0;
 #pragma unroll
   for (int b = 0; b < kSmallBlocks; ++b) base += b < rank ? totals_of[b] : 0;
+  if (base < 0 || base + totals_of[rank] > n) {  // the same in every thread of the block
+    if (tid == 0) set_error(err, CRYS_DEV_BOUNDS);
+    return;
+  }
   if (rank == kSmallBlocks - 1 && tid == 0) *count = static_cast<long long>(base) + totals_of[rank];
   int run = base + wtot[warp];
 #pragma unroll
@@ -630,9 +637,11 @@ extern "C" int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, 
   uint64_t stall_ns = kWaitBoundNs;
   const bool stalled = n > 0 && lo <= hi && order_preserving && take_stall(CRYS_OP_SELECT, &stall_base, &stall_ns);
   if (n > 0 && n <= (order_preserving ? kSmallRows : kSmallRowsAnyOrder) && lo <= hi && !stalled) {
+    int32_t* err = device_error_word();
+    if (!err) return CRYS_ECUDA;
     select_small_kernel<<<kSmallBlocks, kSmallThreads, 0, s>>>(x, static_cast<int>(n), lo,
                                                               static_cast<uint32_t>(hi) - static_cast<uint32_t>(lo), out,
-                                                              reinterpret_cast<long long*>(d_count));
+                                                              reinterpret_cast<long long*>(d_count), err);
     note_launch();
     return check_launch();
   }
