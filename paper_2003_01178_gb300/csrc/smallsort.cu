@@ -268,6 +268,7 @@ __global__ void __launch_bounds__(kThreads, 2) small_sort_kernel(const __grid_co
         local_sort_bucket(l, sh.local, begin, size, parity);
         parity ^= 1u;
       }
+      fence_proxy_async_smem();  // the next bucket's values come by a bulk copy into the same place
       __syncthreads();  // the bucket is stored: its shared memory is free
     }
     return;
