@@ -300,6 +300,7 @@ __device__ void scan_tiles(const SelectArgs& a, OrderedShared& sh, int64_t ntile
       }
       // this chunk's turn: the critical section is one shared-memory read and one write
       __threadfence_block();
+      __syncwarp();  // lane 0 saw the turn: its fence orders every lane's read
       const uint64_t base = sh.running;  // written before the turn was passed on
       __syncwarp();
       if (there == kChunk && lane == 0) {

@@ -365,15 +365,18 @@ __device__ void scan_tiles(const PassArgs& a, int scanner, int64_t tiles, ScanSh
         continue;
       }
       __threadfence_block();
+      __syncwarp();  // lane 0 saw the turn: its fence orders every lane's read
       uint32_t run = running[lane];
       if (there == chunk) {  // the turn goes on before the stores
         uint32_t total = 0;
 #pragma unroll
         for (int r = 0; r < kScanTiles; ++r) total += w[r] & kValueMask;
         running[lane] = run + total;
-        __threadfence_block();
         __syncwarp();
-        if (lane == 0) *turn = c + 1;
+        if (lane == 0) {
+          __threadfence_block();  // after every lane's sum
+          *turn = c + 1;
+        }
       }
 #pragma unroll
       for (int r = 0; r < kScanTiles; ++r) {
