@@ -494,8 +494,10 @@ __global__ void __launch_bounds__(THREADS + 2 * kWarp) select_ordered_kernel(Sel
 // No scratch and no cleared counter, so the call is one launch; it is launches that bound
 // small calls (100,003 rows: 11.8 us per call with two clearings and the tiled kernel, 6.2 us
 // with this one).  The line is what 8 blocks hold in registers, 16 rows per thread; without an
-// order half of that, for the tiled kernel needs one clearing less there (all of 65536 rows 6.3
-// against 6.8 us, all of 131072 rows 8.2 against 6.5).
+// order half of that, for the tiled kernel needs one clearing less there (three quarters and
+// all of 65536 rows 6.2 against 6.5 us, of 131072 rows 8.2 against 6.3).  The values go through
+// shared memory so that a warp's stores are consecutive: stored from the registers, all of
+// 65536 rows took 7.7 us.
 constexpr int kSmallBlocks = 8;
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallVec = 4;  // groups of 4 rows per thread
@@ -508,6 +510,8 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
   namespace cg = cooperative_groups;
   cluster_arrive_relaxed();  // this block runs; waited for before the first store to another block
   constexpr int WARPS = kSmallThreads / kWarp;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  auto kept = reinterpret_cast<int32_t(*)[128 * kSmallVec]>(smem_raw);  // per warp
   __shared__ int32_t wtot[WARPS];
   __shared__ int32_t totals_of[kSmallBlocks];  // every block's count, written by that block
   cg::cluster_group cluster = cg::this_cluster();
@@ -539,13 +543,9 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
       bits |= static_cast<uint32_t>(hit) << (4 * j + e);
     }
   }
-  // one warp scan of the lanes' counts of all groups (group j's in byte j), then the warps'
-  uint32_t packed = 0;
-#pragma unroll
-  for (int j = 0; j < kSmallVec; ++j) packed |= static_cast<uint32_t>(__popc((bits >> (4 * j)) & 0xFu)) << (8 * j);
-  const uint32_t incl = static_cast<uint32_t>(warp_inclusive_scan(static_cast<int32_t>(packed), lane));
-  const uint32_t excl = incl - packed, totals = __shfl_sync(0xFFFFFFFFu, incl, kWarp - 1);
-  if (lane == 0) wtot[warp] = static_cast<int32_t>((totals & 0xFFu) + ((totals >> 8) & 0xFFu) + ((totals >> 16) & 0xFFu) + (totals >> 24));
+  // the warp's selected values to its own part of shared memory, then one scan of the warps
+  const int run = compact_warp<4 * kSmallVec>(v, bits, kept[warp]);
+  if (lane == 0) wtot[warp] = run;
   __syncthreads();
   cluster_wait();  // every block runs: their shared memory may be written
   if (warp == 0) {
@@ -564,15 +564,8 @@ __global__ void __cluster_dims__(kSmallBlocks, 1, 1) __launch_bounds__(kSmallThr
     return;
   }
   if (rank == kSmallBlocks - 1 && tid == 0) *count = static_cast<long long>(base) + totals_of[rank];
-  int run = base + wtot[warp];
-#pragma unroll
-  for (int j = 0; j < kSmallVec; ++j) {
-    int pos = run + static_cast<int>((excl >> (8 * j)) & 0xFFu);
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-      if (bits & (1u << (4 * j + e))) out[pos++] = v[4 * j + e];
-    run += static_cast<int>((totals >> (8 * j)) & 0xFFu);
-  }
+  int32_t* dst = out + base + wtot[warp];
+  for (int i = lane; i < run; i += kWarp) dst[i] = kept[warp][i];
 }
 
 template <int THREADS, int ITEMS>
@@ -640,7 +633,9 @@ extern "C" int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, 
   if (n > 0 && n <= (order_preserving ? kSmallRows : kSmallRowsAnyOrder) && lo <= hi && !stalled) {
     int32_t* err = device_error_word();
     if (!err) return CRYS_ECUDA;
-    select_small_kernel<<<kSmallBlocks, kSmallThreads, 0, s>>>(x, static_cast<int>(n), lo,
+    constexpr size_t smem = sizeof(int32_t) * 4 * kSmallVec * kSmallThreads;
+    if (!allow_smem(select_small_kernel, smem)) return CRYS_ECUDA;
+    select_small_kernel<<<kSmallBlocks, kSmallThreads, smem, s>>>(x, static_cast<int>(n), lo,
                                                               static_cast<uint32_t>(hi) - static_cast<uint32_t>(lo), out,
                                                               reinterpret_cast<long long*>(d_count), err);
     note_launch();

@@ -42,3 +42,24 @@ def test_small_selects_beside_other_work(crys, n):
     torch.cuda.synchronize()
     for i, (out, c) in enumerate(zip(outs, counts.tolist())):
         assert c == refs[i % 8].numel() and torch.equal(out[:c], refs[i % 8]), i
+
+
+@pytest.mark.parametrize("off", [0, 1, 2, 3])
+@pytest.mark.parametrize("n", [3, 4, 5, 4099, 65_536, 131_072])
+def test_small_selects_of_most_rows(crys, n, off):
+    # everything selected, and all but rows at every place of a group of four; outputs that start
+    # at any element
+    x = torch.arange(n, dtype=torch.int32, device="cuda")
+    for gap in (0, 5, 64, 1021):
+        if gap:
+            x[::gap] = -1
+        ref = x[x >= 0]
+        buf = torch.full((n + 8,), 777, dtype=torch.int32, device="cuda")
+        count = torch.zeros(1, dtype=torch.int64, device="cuda")
+        tb = crys.crys_select(None, n, 0, I32_MAX, None, None, 1, None, -1)
+        temp = crys.scratch(tb, "cuda")
+        crys.crys_select(x, n, 0, I32_MAX, buf[off:off + n], count, 1, temp, tb)
+        c = int(count.item())
+        assert c == ref.numel() and torch.equal(buf[off:off + c], ref)
+        assert bool((buf[:off] == 777).all()) and bool((buf[off + c:] == 777).all())
+        x = torch.arange(n, dtype=torch.int32, device="cuda")
