@@ -22,7 +22,7 @@ struct KeyRange {
 };
 
 constexpr int kRangeThreads = 1024;
-constexpr int kRangeSamples = 8;  // per thread
+constexpr int kRangeBatch = 8;  // samples of a thread in flight together
 // Keys that differ in at most this many bytes are sorted stably by digits, one pass per byte
 // (and a count of 0.2 ms for 2^28 rows): two passes for 2^28 keys of two bytes take 3.09 ms, the
 // buckets 4.8 ms when their leading bits are spread evenly; three passes for keys of three
@@ -30,30 +30,51 @@ constexpr int kRangeSamples = 8;  // per thread
 // a bucket.  A fourth pass would add 1.2 to 1.4 ms, to more than the 4.36 ms of the buckets.
 constexpr int kFewBytes = 3;
 
-// One block: 256 runs of 32 consecutive keys, spread evenly over the column and taken by a
-// warp each, always with the first and the last key.  `few`, when given, is set if the sampled
-// keys differ in at most kFewBytes of their bytes.
+// Rows sampled: the power of two of at least 2 sqrt(n), at most 8192.
+inline int range_samples(int64_t n) {
+  int samples = kRangeThreads;
+  while (samples < 8192 && static_cast<int64_t>(samples) * samples < 4 * n) samples *= 2;
+  return samples;
+}
+
+// Row of sample i: the first, the last, then rows drawn independently (the 32-bit finaliser of
+// MurmurHash3, Appleby).  Not evenly spaced runs of rows: where a column is made of pieces with
+// ranges of their own, those runs miss whole pieces, and all keys of a missed one beyond the
+// sampled range go to one bucket (MSB sort of 2^28 keys in 1000 such pieces: 17.9 ms).
+__device__ __forceinline__ int64_t sample_row(uint32_t i, int64_t n) {
+  if (i < 2) return i == 0 ? 0 : n - 1;
+  uint32_t h = i * 0x9E3779B9u;
+  h ^= h >> 16;
+  h *= 0x85EBCA6Bu;
+  h ^= h >> 13;
+  h *= 0xC2B2AE35u;
+  h ^= h >> 16;
+  return static_cast<int64_t>((static_cast<uint64_t>(h) * static_cast<uint64_t>(n)) >> 32);
+}
+
+// One block.  `few`, when given, is set if the sampled keys differ in at most kFewBytes of their
+// bytes.
 static __global__ void __launch_bounds__(kRangeThreads) key_range_kernel(const int32_t* __restrict__ keys, int64_t n,
-                                                                         int bits, KeyRange* out, uint32_t* few) {
+                                                                         int bits, int samples, KeyRange* out, uint32_t* few) {
   __shared__ int32_t slo[kRangeThreads / kWarp], shi[kRangeThreads / kWarp];
   __shared__ uint32_t sdiff[kRangeThreads / kWarp];
   const int lane = threadIdx.x % kWarp, warp = threadIdx.x / kWarp;
-  constexpr int kRuns = kRangeThreads / kWarp * kRangeSamples;
-  int32_t k[kRangeSamples];
-#pragma unroll
-  for (int j = 0; j < kRangeSamples; ++j) {
-    const int64_t run = static_cast<int64_t>(j) * (kRangeThreads / kWarp) + warp;
-    const int64_t i = run * (n > kWarp ? n - kWarp : 0) / (kRuns - 1) + lane;
-    k[j] = keys[i < n ? i : n - 1];
-  }
   const int32_t ref = keys[0];
-  int32_t lo = k[0], hi = k[0];
-  uint32_t diff = static_cast<uint32_t>(k[0] ^ ref);
+  int32_t lo = ref, hi = ref;
+  uint32_t diff = 0;
+  for (int i0 = threadIdx.x; i0 < samples; i0 += kRangeBatch * kRangeThreads) {
+    int32_t k[kRangeBatch];
 #pragma unroll
-  for (int j = 1; j < kRangeSamples; ++j) {
-    lo = min(lo, k[j]);
-    hi = max(hi, k[j]);
-    diff |= static_cast<uint32_t>(k[j] ^ ref);
+    for (int j = 0; j < kRangeBatch; ++j) {
+      const int i = i0 + j * kRangeThreads;
+      k[j] = i < samples ? keys[sample_row(static_cast<uint32_t>(i), n)] : ref;
+    }
+#pragma unroll
+    for (int j = 0; j < kRangeBatch; ++j) {
+      lo = min(lo, k[j]);
+      hi = max(hi, k[j]);
+      diff |= static_cast<uint32_t>(k[j] ^ ref);
+    }
   }
   lo = __reduce_min_sync(0xFFFFFFFFu, lo);
   hi = __reduce_max_sync(0xFFFFFFFFu, hi);
@@ -70,8 +91,8 @@ static __global__ void __launch_bounds__(kRangeThreads) key_range_kernel(const i
     hi = max(hi, shi[w]);
     diff |= sdiff[w];
   }
-  // the extremes of 8192 sampled keys of an even distribution miss about 2^-13 of it at
-  // either end, eight buckets of 65536: widened by 2^-8 of the range they miss nothing
+  // the extremes of 1024 to 8192 sampled keys of an even distribution miss 2^-10 to 2^-13 of it
+  // at either end: widened by 2^-8 of the range they miss nothing
   const int64_t widen = (static_cast<int64_t>(hi) - lo) / 256;
   const int64_t l = max(static_cast<int64_t>(lo) - widen, static_cast<int64_t>(INT32_MIN));
   const int64_t h = min(static_cast<int64_t>(hi) + widen, static_cast<int64_t>(INT32_MAX));
@@ -86,7 +107,7 @@ static __global__ void __launch_bounds__(kRangeThreads) key_range_kernel(const i
 }
 
 inline int launch_key_range(const int32_t* keys, int64_t n, int bits, KeyRange* out, uint32_t* few, cudaStream_t s) {
-  key_range_kernel<<<1, kRangeThreads, 0, s>>>(keys, n, bits, out, few);
+  key_range_kernel<<<1, kRangeThreads, 0, s>>>(keys, n, bits, range_samples(n), out, few);
   note_launch();
   return check_launch();
 }
