@@ -8,7 +8,8 @@
 //    ranges fill the buckets too.  One kernel reads the keys and counts all buckets, which
 //    gives the passes' bucket starts and shows whether any bucket is too large for a block.
 //  * digits: when one is (heavily repeated or clustered keys), when a sample of the keys differs
-//    in at most three bytes (keyrange.cuh), or when there are too many rows, the
+//    in at most three bytes or shows more than eight rows per key value (keyrange.cuh), or
+//    when there are too many rows, the
 //    least-significant-digit sort: 8-bit digits, a stable pass per digit from the low one to
 //    the high one.  Digits that have one value in all keys are skipped.
 //
@@ -53,7 +54,7 @@ struct SortHead {
   unsigned int abort_word;   // set by the first block of this sort that gives up
   unsigned int counted;      // blocks of the counting kernels that have finished
   unsigned int digits_counted;
-  unsigned int crowded;      // a bucket is too large for a block, or the keys differ in few bytes
+  unsigned int crowded;      // a bucket is too large for a block, or the keys are few (keyrange.cuh)
   uint32_t buckets;          // 1: sorted by buckets, 0: by digits
   uint32_t passes;           // passes that do work; pass j writes to the output when an even number follows
   KeyRange range;
