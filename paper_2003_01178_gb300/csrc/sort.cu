@@ -390,13 +390,16 @@ __device__ void scan_tiles(const PassArgs& a, int scanner, int64_t tiles, ScanSh
 }
 
 // This tile's rows of one digit: counted in the tiles before it.  False when that never came.
-__device__ __forceinline__ bool prefix_of(const PassArgs& a, const uint32_t* word, uint32_t* excl) {
+// The word is cleared for the next pass: its scanner is done with it once the prefix is
+// there, and nobody else reads it.
+__device__ __forceinline__ bool prefix_of(const PassArgs& a, uint32_t* word, uint32_t* excl) {
   SpinGuard guard;
   uint32_t w = ld_relaxed_u32(word);
   while ((w >> 30) != 2u) {
     if (!guard.go_on(&a.head->abort_word, a.wait_ns, a.err)) return false;
     w = ld_relaxed_u32(word);
   }
+  st_relaxed_u32(word, 0u);
   *excl = w & kValueMask;
   return true;
 }
@@ -594,7 +597,6 @@ int run_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out, 
   const size_t smem = static_cast<size_t>(TILE) * 8;
   auto kernel = sort_pass_kernel<THREADS, ITEMS>;
   if (!allow_smem(kernel, smem)) return CRYS_ECUDA;
-  if (cudaMemsetAsync(temp + L.hist, 0, L.status - L.hist, s) != cudaSuccess) return CRYS_ECUDA;
   SortHead* head = reinterpret_cast<SortHead*>(temp + L.counters);
   uint32_t* base = reinterpret_cast<uint32_t*>(temp + L.base);
   int32_t* err = device_error_word();
@@ -602,8 +604,12 @@ int run_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out, 
   const int bits = n <= kMaxBucketRows ? range_bits(n, kLocalCap) : 0;
   uint32_t* counts = bits ? bucket_words(temp, L, bits, tiles) : nullptr;
   const int64_t buckets = int64_t{1} << bits;
+  // One clearing: the histogram, the head, the status words (every tile of a pass clears its
+  // own again) and, right behind them, the counts of more than 256 buckets.
+  size_t cleared = L.status + up256(static_cast<size_t>(tiles) * kRadix * 4) - L.hist;
+  if (counts && bits > 8) cleared += static_cast<size_t>(buckets) * 4;
+  if (cudaMemsetAsync(temp + L.hist, 0, cleared, s) != cudaSuccess) return CRYS_ECUDA;
   if (counts) {
-    if (bits > 8 && cudaMemsetAsync(counts, 0, static_cast<size_t>(buckets) * 4, s) != cudaSuccess) return CRYS_ECUDA;
     if (launch_key_range(keys_in, n, bits, &head->range, &head->crowded, s) != CRYS_OK) return CRYS_ECUDA;
     const size_t bins = static_cast<size_t>(buckets) * 2;
     if (!allow_smem(count_buckets_kernel, size_t{2} << 16)) return CRYS_ECUDA;
@@ -636,8 +642,6 @@ int run_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out, 
     a.wait_ns = p == 0 ? stall_ns : kWaitBoundNs;
     a.pass = p;
     a.digit_base = base + p * kRadix;
-    if (cudaMemsetAsync(a.status, 0, static_cast<size_t>(tiles) * kRadix * 4, s) != cudaSuccess)
-      return CRYS_ECUDA;
     kernel<<<static_cast<unsigned int>(tiles + kScanners), THREADS, smem, s>>>(a);
     note_launch();
     if (check_launch() != CRYS_OK) return CRYS_ECUDA;
