@@ -502,15 +502,17 @@ def frac(alg_bytes, ms):
 
 def autotune(op, launch, args):
     """Pick the tile shape of `op` on this workload (crys_tile_variants x timing) unless
-    --no-tune; returns the chosen (threads, items) and the median ms of every variant."""
+    --no-tune; returns the (threads, items) that was set, or "chosen per call" when the library's
+    own choice is as fast, and the median ms of every variant and of that choice."""
     import paper_2003_01178_gb300 as crys
     from paper_2003_01178_gb300 import tuner
     times = {}
     if not args.no_tune:
         res = tuner.tune(op, launch, reps=3, warmup=1)
         times = {f"{v['threads']}x{v['items']}": round(v["ms"], 4) for v in res["variants"].values()}
-    v = crys.crys_get_tile(op)
-    return {"shape": list(crys.crys_tile_variants(op)[v]), "variants_ms": times}
+        times["chosen per call"] = round(res["own_ms"], 4)
+    shape = list(crys.crys_tile_variants(op)[crys.crys_get_tile(op)]) if crys.crys_tile_is_set(op) else "chosen per call"
+    return {"shape": shape, "variants_ms": times}
 
 
 def time_launches(fn, steps, warmup, stream, flush=None):

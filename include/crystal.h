@@ -382,6 +382,11 @@ int crys_tagged_launch(const void* dev_block, crys_stream s);
  * Each operator is compiled for several tile shapes (threads per block x items per
  * thread, Section 3.3).  crys_tile_variants lists them; crys_set_tile picks the one
  * used by later calls in this process (an autotuner sweeps and persists the choice).
+ * While none was set, or after crys_reset_tile, an operator chooses for each call:
+ * variant 0 but for the sizes and plans where something else was measured faster - another
+ * variant (CRYS_OP_PROBE, CRYS_OP_PLAN), or for few rows one launch that has no tiles
+ * (CRYS_OP_SELECT up to 131072 rows, 65536 without an order; CRYS_OP_SORT up to 2^20
+ * rows).  A variant that was set is used for every size.
  * CRYS_OP_SHARED_SCAN is crys_run_plans (also when crys_run_plans_tagged falls back to
  * it); CRYS_OP_TAGGED_SCAN is the tagged scan of crys_run_plans_tagged and of the
  * replayable launch (a block must be launched under the shape it was prepared for). */
@@ -396,7 +401,9 @@ int crys_tagged_launch(const void* dev_block, crys_stream s);
 /* Writes up to `max` (threads, items) pairs; returns the number of variants (or <0). */
 int crys_tile_variants(int op, int32_t* threads, int32_t* items, int32_t max);
 int crys_set_tile(int op, int32_t variant);
-int crys_get_tile(int op);
+int crys_reset_tile(int op);
+int crys_get_tile(int op);    /* the variant that was set, 0 if none was */
+int crys_tile_is_set(int op); /* 1 if one was, 0 if not */
 
 #ifdef __cplusplus
 }

@@ -120,6 +120,8 @@ def lib():
         L.crys_tile_variants.argtypes = [C.c_int, C.POINTER(C.c_int32), C.POINTER(C.c_int32), i32]
         L.crys_set_tile.argtypes = [C.c_int, i32]
         L.crys_get_tile.argtypes = [C.c_int]
+        L.crys_reset_tile.argtypes = [C.c_int]
+        L.crys_tile_is_set.argtypes = [C.c_int]
         for fn in ("crys_device_errors", "crys_debug_stall", "crys_select", "crys_select_static", "crys_select_strawman",
                    "crys_project", "crys_hash_init",
                    "crys_hash_build", "crys_probe_aggregate", "crys_sort", "crys_sort_msb",
@@ -128,7 +130,7 @@ def lib():
                    "crys_run_plan", "crys_run_plans", "crys_run_plans_tagged_bytes",
                    "crys_run_plans_tagged", "crys_tagged_block_bytes", "crys_tagged_prepare",
                    "crys_tagged_launch", "crys_tile_variants", "crys_set_tile",
-                   "crys_get_tile"):
+                   "crys_get_tile", "crys_reset_tile", "crys_tile_is_set"):
             getattr(L, fn).restype = C.c_int
         _lib = L
     return _lib
@@ -357,8 +359,21 @@ def crys_set_tile(op: int, variant: int) -> None:
     _check(lib().crys_set_tile(op, variant), "crys_set_tile")
 
 
+def crys_reset_tile(op: int) -> None:
+    """Leaves the choice of `op`'s tile shape to the library again, call by call."""
+    _check(lib().crys_reset_tile(op), "crys_reset_tile")
+
+
 def crys_get_tile(op: int) -> int:
     return int(lib().crys_get_tile(op))
+
+
+def crys_tile_is_set(op: int) -> bool:
+    """Whether later calls of `op` use a shape that was set; otherwise the library chooses."""
+    r = int(lib().crys_tile_is_set(op))
+    if r < 0:
+        raise CrystalError(r, "crys_tile_is_set")
+    return r == 1
 
 
 # ---------------------------------------------------------------- conveniences

@@ -19,6 +19,7 @@ std::mutex g_mutex;
 int32_t* g_error_ptr[kMaxDevices] = {};
 int g_sms[kMaxDevices] = {};
 std::atomic<int64_t> g_launches{0};
+// Tile variant of each operator plus one; 0: none was set.
 std::atomic<int> g_variant[CRYS_NUM_OPS] = {};
 // pending crys_debug_stall request (op, first tile, wait bound), taken by the next call
 std::mutex g_stall_mutex;
@@ -113,8 +114,13 @@ bool take_stall(int op, uint32_t* first_tile, uint64_t* wait_ns) {
 }
 
 int tile_variant(int op) {
-  if (op < 0 || op >= CRYS_NUM_OPS) return 0;
-  return g_variant[op].load(std::memory_order_relaxed);
+  const int v = set_tile_variant(op);
+  return v < 0 ? 0 : v;
+}
+
+int set_tile_variant(int op) {
+  if (op < 0 || op >= CRYS_NUM_OPS) return -1;
+  return g_variant[op].load(std::memory_order_relaxed) - 1;
 }
 
 }  // namespace crys
@@ -173,13 +179,24 @@ int crys_tile_variants(int op, int32_t* threads, int32_t* items, int32_t max) {
 int crys_set_tile(int op, int32_t variant) {
   if (op < 0 || op >= CRYS_NUM_OPS || variant < 0 || variant >= crys::kNumVariants[op])
     return CRYS_EINVAL;
-  crys::g_variant[op].store(variant);
+  crys::g_variant[op].store(variant + 1);
+  return CRYS_OK;
+}
+
+int crys_reset_tile(int op) {
+  if (op < 0 || op >= CRYS_NUM_OPS) return CRYS_EINVAL;
+  crys::g_variant[op].store(0);
   return CRYS_OK;
 }
 
 int crys_get_tile(int op) {
   if (op < 0 || op >= CRYS_NUM_OPS) return CRYS_EINVAL;
-  return crys::g_variant[op].load();
+  return crys::tile_variant(op);
+}
+
+int crys_tile_is_set(int op) {
+  if (op < 0 || op >= CRYS_NUM_OPS) return CRYS_EINVAL;
+  return crys::set_tile_variant(op) >= 0 ? 1 : 0;
 }
 
 }  // extern "C"

@@ -340,7 +340,7 @@ int crys_probe_aggregate(const int32_t* fk, const int32_t* payload, int64_t n, c
       // 0.553, 1.021 and 0.962 with 256 x 8; of 1 MB 0.985 and 0.913; 2^24 probes of 64 and 512
       // KB 42.0 and 68.9 us against 39.3 and 66.2).
       static_assert(kTiles[kOp][1].threads == 256 && kTiles[kOp][1].items == 16, "the larger tiles");
-      if (a.table_slots == 0 && ht->capacity * 8 <= 16 * kSmemTableBytes && n >= (1 << 25))
+      if (set_tile_variant(kOp) < 0 && a.table_slots == 0 && ht->capacity * 8 <= 16 * kSmemTableBytes && n >= (1 << 25))
         return launch_probe<kTiles[kOp][1].threads, kTiles[kOp][1].items>(a, s);
       return launch_probe<kTiles[kOp][0].threads, kTiles[kOp][0].items>(a, s);
   }

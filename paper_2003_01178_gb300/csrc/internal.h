@@ -17,8 +17,11 @@ void note_launch(int kernels = 1);
 // Number of SMs of the current device.
 int sm_count();
 
-// Current tile variant of an operator (index into its variant table).
+// Tile variant of an operator (index into its variant table): the one that was set, or 0.
 int tile_variant(int op);
+
+// The variant that was set, or -1: then the operator is free to choose by the call's sizes.
+int set_tile_variant(int op);
 
 // The stall requested by crys_debug_stall for the next call of `op`, consumed by this
 // call: tile ids start at *first_tile and look-back waits give up after *wait_ns.

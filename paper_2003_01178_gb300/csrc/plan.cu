@@ -1852,13 +1852,13 @@ bool of_fixed_shape(const DevQuery& q) {
          (q.agg_op == CRYS_AGG_A_MUL_B || q.agg_op == CRYS_AGG_A);
 }
 
-// The default shape takes its smaller tiles for any plan while these are at most one per SM: half
+// Without a shape set, any plan takes the smaller tiles while these are at most one per SM: half
 // as many larger ones leave the other SMs idle (three joins on direct tables, 100,003 rows: 6.4
 // us with 256 x 8, 7.9 with 512 x 8; 311,296 rows 6.5 and 7.9; 400,003 rows, on more than one
 // tile for some SMs, 8.2 and 8.0).
 bool one_small_tile_per_sm(int64_t rows) { return rows <= static_cast<int64_t>(sm_count()) * 256 * 8; }
 
-// Rows up to which the default shape takes its smaller tiles for plans of the Q1 family: the
+// Rows up to which, without a shape set, plans of the Q1 family take the smaller tiles: the
 // last tiles of so few rows leave much of the chip idle (12,000,001 rows 31.4 us with 256 x 8,
 // 32.9 with 512 x 8; 17,000,003 rows 43.2 and 43.5; 2^25 rows 80.4 and 79.5).
 constexpr int64_t kSmallTileRows = int64_t{3} << 23;
@@ -2464,7 +2464,8 @@ int crys_run_plan(const crys_table* fact, const crys_plan* plan, crys_stream str
     case 3: return launch_plan<kTiles[kOp][3].threads, kTiles[kOp][3].items>(a, s);
     default:
       static_assert(kTiles[kOp][1].threads == 256 && kTiles[kOp][1].items == 8, "the default shape's smaller tiles");
-      if (one_small_tile_per_sm(fact->n_rows) || (fact->n_rows <= kSmallTileRows && of_fixed_shape(a.q)))
+      if (set_tile_variant(kOp) < 0 &&
+          (one_small_tile_per_sm(fact->n_rows) || (fact->n_rows <= kSmallTileRows && of_fixed_shape(a.q))))
         return launch_plan<kTiles[kOp][1].threads, kTiles[kOp][1].items>(a, s);
       return launch_plan<kTiles[kOp][0].threads, kTiles[kOp][0].items>(a, s);
   }

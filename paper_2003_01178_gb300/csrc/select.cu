@@ -630,7 +630,8 @@ extern "C" int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, 
   uint32_t stall_base = 0;
   uint64_t stall_ns = kWaitBoundNs;
   const bool stalled = n > 0 && lo <= hi && order_preserving && take_stall(CRYS_OP_SELECT, &stall_base, &stall_ns);
-  if (n > 0 && n <= (order_preserving ? kSmallRows : kSmallRowsAnyOrder) && lo <= hi && !stalled) {
+  const bool any_tile = set_tile_variant(kOp) < 0;
+  if (n > 0 && n <= (order_preserving ? kSmallRows : kSmallRowsAnyOrder) && lo <= hi && !stalled && any_tile) {
     int32_t* err = device_error_word();
     if (!err) return CRYS_ECUDA;
     constexpr size_t smem = sizeof(int32_t) * 4 * kSmallVec * kSmallThreads;

@@ -688,17 +688,18 @@ extern "C" int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t
   uint64_t stall_ns = kWaitBoundNs;
   // a test's stall applies to the first pass: a stalled sort goes by passes (one block has no tiles)
   const bool stalled = take_stall(CRYS_OP_SORT, &stall_base, &stall_ns);
-  if (n <= kLocalCap) {  // one block sorts everything
+  const bool any_tile = set_tile_variant(kOp) < 0;
+  if (n <= kLocalCap && any_tile) {  // one block sorts everything
     int32_t* err = device_error_word();
     if (!err) return CRYS_ECUDA;
     return launch_local_sort<false>(
         LocalArgs{keys_in, vals_in, keys_out, vals_out, nullptr, nullptr, static_cast<uint32_t>(n), err}, 1, s);
   }
-  if (!stalled && small_sort_fits(n))
+  if (!stalled && any_tile && small_sort_fits(n))
     return launch_small_sort(keys_in, vals_in, reinterpret_cast<int32_t*>(temp + L.tmp_keys),
                              reinterpret_cast<int32_t*>(temp + L.tmp_vals), keys_out, vals_out, n, temp + L.counters, s);
   // up to 2^20 rows (one pass by buckets) the smallest tile, so that more SMs have one
-  switch (n <= (1 << 20) ? kNumVariants[kOp] - 1 : tile_variant(kOp)) {
+  switch (any_tile && n <= (1 << 20) ? kNumVariants[kOp] - 1 : tile_variant(kOp)) {
     case 1: return run_sort<kTiles[kOp][1].threads, kTiles[kOp][1].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, stall_base, stall_ns, s);
     case 2: return run_sort<kTiles[kOp][2].threads, kTiles[kOp][2].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, stall_base, stall_ns, s);
     case 3: return run_sort<kTiles[kOp][3].threads, kTiles[kOp][3].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, stall_base, stall_ns, s);

@@ -2,10 +2,13 @@
 
 Each operator is compiled for a few tile shapes (``crys_tile_variants``).  ``tune`` times
 every variant of an operator on a caller-supplied launch (CUDA events, warm-up first,
-median of several runs) and selects the fastest with ``crys_set_tile``; ``save`` / ``load``
-persist the choice per device name as JSON so later processes start with it.  The choice
-is stored as the tile shape, not the variant's index, so a library whose variant list
-changed still finds it (or ignores it when that shape is no longer compiled).
+median of several runs), and the library's own choice, which goes by the sizes of a call and
+is not always one of the shapes.  The fastest variant is set with ``crys_set_tile`` where it
+beats that choice by more than repeated runs differ; otherwise the choice stays the
+library's.  ``save`` / ``load`` persist the shapes that are set, per device name as JSON, so
+later processes start with them.  A shape is stored as such, not as the variant's index, so a
+library whose variant list changed still finds it (or ignores it when that shape is no
+longer compiled).
 """
 from __future__ import annotations
 
@@ -15,8 +18,9 @@ import statistics
 
 import torch
 
-from . import OP_NAMES, crys_get_tile, crys_set_tile, crys_tile_variants
+from . import OP_NAMES, crys_get_tile, crys_reset_tile, crys_set_tile, crys_tile_is_set, crys_tile_variants
 
+MARGIN = 0.98   # a variant is set when it takes less than this share of the library's own choice
 DEFAULT_PATH = os.path.join(os.path.expanduser("~"), ".cache", "crystal_gb300_tiles.json")
 
 
@@ -37,14 +41,20 @@ def time_variant(launch, reps: int = 5, warmup: int = 2, stream=None) -> float:
 
 
 def tune(op: int, launch, reps: int = 5, warmup: int = 2) -> dict:
-    """Times every tile variant of `op` on `launch()`; selects and returns the best."""
+    """Times every tile variant of `op` on `launch()`, and the library's own choice; sets the best
+    variant unless that choice is as fast.  "best" is the fastest variant either way."""
+    crys_reset_tile(op)
+    own_ms = time_variant(launch, reps, warmup)
     results = {}
     for v, (threads, items) in enumerate(crys_tile_variants(op)):
         crys_set_tile(op, v)
         results[v] = {"threads": threads, "items": items, "ms": time_variant(launch, reps, warmup)}
     best = min(results, key=lambda v: results[v]["ms"])
-    crys_set_tile(op, best)
-    return {"op": OP_NAMES[op], "best": best, "variants": results}
+    if results[best]["ms"] < MARGIN * own_ms:
+        crys_set_tile(op, best)
+    else:
+        crys_reset_tile(op)
+    return {"op": OP_NAMES[op], "best": best, "set": crys_tile_is_set(op), "own_ms": own_ms, "variants": results}
 
 
 def _key() -> str:
@@ -56,7 +66,8 @@ def save(path: str = DEFAULT_PATH) -> None:
     if os.path.exists(path):
         with open(path) as f:
             data = json.load(f)
-    data[_key()] = {OP_NAMES[op]: list(crys_tile_variants(op)[crys_get_tile(op)]) for op in range(len(OP_NAMES))}
+    data[_key()] = {OP_NAMES[op]: list(crys_tile_variants(op)[crys_get_tile(op)]) for op in range(len(OP_NAMES))
+                    if crys_tile_is_set(op)}
     os.makedirs(os.path.dirname(path), exist_ok=True)
     with open(path, "w") as f:
         json.dump(data, f, indent=1)
