@@ -686,10 +686,10 @@ extern "C" int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t
   char* temp = static_cast<char*>(d_temp);
   uint32_t stall_base = 0;
   uint64_t stall_ns = kWaitBoundNs;
-  // a test's stall applies to the first pass: a stalled sort goes by passes (one block has no tiles)
+  // a test's stall applies to the first pass: a stalled sort goes by passes, whatever its size
   const bool stalled = take_stall(CRYS_OP_SORT, &stall_base, &stall_ns);
   const bool any_tile = set_tile_variant(kOp) < 0;
-  if (n <= kLocalCap && any_tile) {  // one block sorts everything
+  if (n <= kLocalCap && any_tile && !stalled) {  // one block sorts everything
     int32_t* err = device_error_word();
     if (!err) return CRYS_ECUDA;
     return launch_local_sort<false>(
