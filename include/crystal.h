@@ -18,6 +18,9 @@
  *    hash table, a reserved or duplicate key, a group code out of range) set sticky
  *    bits in a per-device error word read with crys_device_errors(); the kernels
  *    never trap, and a kernel that detects one of these stops its own work early.
+ *  - An ordered selection needs room for two of its blocks at a time to advance, a pass of
+ *    the stable sort for nine (eight scan the counts of the others).  Other work that leaves
+ *    less delays the call; only after 60 s without room does it give up (CRYS_DEV_TIMEOUT).
  *  - n == 0 is legal everywhere and produces empty / zero results.
  *  - Scratch: calls that need scratch take (void* d_temp, size_t* temp_bytes).  With
  *    d_temp == NULL the call only stores the required size in *temp_bytes and returns

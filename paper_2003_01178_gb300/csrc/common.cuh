@@ -20,6 +20,9 @@ constexpr int kWarp = 32;
 // microseconds; after this bound the waiting thread sets CRYS_DEV_TIMEOUT and its block
 // abandons the work instead of hanging the GPU.
 constexpr uint64_t kWaitBoundNs = 2000000000ull;
+// The same for a wait for work that no block holds yet because the rest of the launch has not
+// started: other work on the GPU may keep it waiting for long without anything being wrong.
+constexpr uint64_t kQueueBoundNs = 60000000000ull;
 constexpr uint64_t kEmptySlot = 0xFFFFFFFFFFFFFFFFull;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
@@ -194,6 +197,30 @@ __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t* p) {
 }
 __device__ __forceinline__ void st_relaxed_u32(uint32_t* p, uint32_t v) {
   asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// The same for a scanner, which waits for a tile's count: `tickets` is the counter that hands
+// the tiles out, and the tile is held by a block once it has reached `held_at`.  Until then the
+// rest of the launch has not started, other work on the GPU may keep it waiting for long, and
+// the wait's bound does not run (kQueueBoundNs does): each look past half the bound asks.  The
+// look is a call, so that the polling loops stay as short as without it (inlined, it made a
+// selection of 2^29 rows 3% slower).
+struct ScanWait {
+  uint64_t t0, first;
+};
+
+static __device__ __noinline__ bool scan_look(ScanWait* w, const uint32_t* tickets, int64_t held_at,
+                                              unsigned int* abort_word, uint64_t wait_ns, int32_t* err) {
+  const uint64_t now = global_timer_ns();
+  if (w->t0 == 0) w->t0 = w->first = now;
+  if (now - w->t0 > wait_ns / 2 && now - w->first < kQueueBoundNs && static_cast<int64_t>(ld_relaxed_u32(tickets)) < held_at)
+    w->t0 = now;
+  if (now - w->t0 > wait_ns) {
+    set_error(err, CRYS_DEV_TIMEOUT);
+    *reinterpret_cast<volatile unsigned int*>(abort_word) = 1u;
+    return false;
+  }
+  return *reinterpret_cast<volatile unsigned int*>(abort_word) == 0u;
 }
 
 // ---------------------------------------------------------------- hashing

@@ -266,7 +266,8 @@ __device__ void scan_tiles(const SelectArgs& a, OrderedShared& sh, int64_t ntile
     uint64_t w[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) w[r] = i0 + r * kWarp < ntiles ? 0ull : kFlagAggregate;
-    SpinGuard guard;
+    ScanWait wait = {};
+    uint32_t spins = 0;
     int handed = 0;  // words of the chunk whose position is out
     int there = 0;   // published words in front of the first missing one
     uint32_t before[R], total = 0;  // their exclusive prefix and sum
@@ -292,10 +293,15 @@ __device__ void scan_tiles(const SelectArgs& a, OrderedShared& sh, int64_t ntile
       }
       const bool mine = __shfl_sync(0xFFFFFFFFu, static_cast<int>(*turn == c), 0) != 0;
       if (there == handed || !mine) {
-        if (!__all_sync(0xFFFFFFFFu, guard.go_on(a.abort_word, a.wait_ns, a.err)) || __any_sync(0xFFFFFFFFu, *gave_up)) {
-          if (lane == 0) *gave_up = 1;
-          return;
+        if (++spins % 32 == 0) {
+          // ids from tile_base on are handed out in order: the first missing tile is among them
+          const int64_t held_at = there < kChunk ? c * kChunk + there + 1 - static_cast<int64_t>(a.tile_base) : 0;
+          if (!__all_sync(0xFFFFFFFFu, scan_look(&wait, a.tile_counter, held_at, a.abort_word, a.wait_ns, a.err))) {
+            if (lane == 0) *gave_up = 1;
+            return;
+          }
         }
+        if (__any_sync(0xFFFFFFFFu, *gave_up)) return;
         continue;
       }
       // this chunk's turn: the critical section is one shared-memory read and one write

@@ -344,7 +344,8 @@ __device__ void scan_tiles(const PassArgs& a, int scanner, int64_t tiles, ScanSh
     uint32_t w[kScanTiles];
 #pragma unroll
     for (int r = 0; r < kScanTiles; ++r) w[r] = 0;
-    SpinGuard guard;
+    ScanWait wait = {};
+    uint32_t spins = 0;
     int handed = 0, there = 0;  // tiles whose prefixes are out; published tiles in front
     while (handed < chunk) {
       if (there < chunk) {
@@ -358,11 +359,16 @@ __device__ void scan_tiles(const PassArgs& a, int scanner, int64_t tiles, ScanSh
       }
       const bool mine = __shfl_sync(0xFFFFFFFFu, static_cast<int>(*turn == c), 0) != 0;
       if (there == handed || !mine) {
-        if (!__all_sync(0xFFFFFFFFu, guard.go_on(&a.head->abort_word, a.wait_ns, a.err)) ||
-            __any_sync(0xFFFFFFFFu, *gave_up)) {
-          if (lane == 0) *gave_up = 1;
-          return;
+        if (++spins % 32 == 0) {
+          // the first kScanners tickets are no tiles, then ids from tile_base on are handed out in order
+          const int64_t held_at = there < chunk ? first + there + 1 + kScanners - static_cast<int64_t>(a.tile_base) : 0;
+          if (!__all_sync(0xFFFFFFFFu, scan_look(&wait, &a.head->tile_counter[a.pass], held_at, &a.head->abort_word,
+                                                 a.wait_ns, a.err))) {
+            if (lane == 0) *gave_up = 1;
+            return;
+          }
         }
+        if (__any_sync(0xFFFFFFFFu, *gave_up)) return;
         continue;
       }
       __threadfence_block();
