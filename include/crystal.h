@@ -200,22 +200,25 @@ int crys_probe_aggregate(const int32_t* fk, const int32_t* payload, int64_t n,
  * then sorted inside one thread block; other keys take a least-significant-digit sort, a
  * pass per 8-bit digit that varies.  The choice is made on the device.  Each pass ranks a
  * tile stably inside the thread block and finds the tile's output offsets with a chained
- * scan over the tiles.  Up to 4992 rows are sorted by one block.  n <= 2^30 - 1.
+ * scan over the tiles.  More than 2^28 rows always take a pass per digit.  Up to 4992 rows
+ * are sorted by one block and up to 2^20 rows by one cooperative launch (while no tile shape
+ * is set).  n <= 2^30 - 1.
  * keys_out/vals_out must not overlap the inputs; the inputs are not modified. */
 int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out,
               int32_t* vals_out, int64_t n, void* d_temp, size_t* temp_bytes, crys_stream s);
 
 /* Most-significant-digit radix sort (Section 4.4: the GPU sort behind the paper's sort
- * figure is an MSB radix sort, not stable).  None, one or two partition passes of at most 8
- * bits (n <= 4992, n <= 2^20, larger), each a histogram, a scan and a scatter whose tiles
- * rank their keys with shared-memory atomics and reserve each digit's run with one global
- * atomic; then every bucket is sorted inside one thread block by its remaining bits and
- * stored.  The passes' bits are those of a key's place between the smallest and the largest
+ * figure is an MSB radix sort, not stable).  Up to 2^20 rows the one launch of crys_sort (if
+ * keys_out is 16-byte aligned; one partition pass if not), above that two partition passes
+ * of at most 8 bits, each a histogram, a scan and a scatter whose tiles rank their keys with
+ * shared-memory atomics and reserve each digit's run with one global atomic; then every
+ * bucket is sorted inside one thread block by its remaining bits and stored.  The passes' bits are those of a key's place between the smallest and the largest
  * key of a sample, so narrow key ranges fill the buckets like wide ones.
  * Keys come out in ascending signed order; rows with EQUAL keys may come out in any order
  * (unstable), so (key, value) pairs are a permutation of the input pairs.  A bucket of
- * more than 4992 rows (heavily repeated or clustered keys) is sorted by one block through
- * global memory: correct for every input, slow only for such skew.  n <= 2^31 - 1; keys_out /
+ * more than 4992 rows (heavily repeated or clustered keys, or more than about 315M rows) is
+ * divided in two where both parts fit a block, and sorted by one block through global memory
+ * otherwise: correct for every input, slow only for such skew.  n <= 2^31 - 1; keys_out /
  * vals_out must not overlap the inputs.  Scratch (two-call size query): n keys + n values
  * plus at most 1.1 MB of bucket arrays. */
 int crys_sort_msb(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out,

@@ -370,8 +370,80 @@ __device__ __forceinline__ void local_sort_bucket(const LocalArgs& a, LocalShare
   }
 }
 
-// One block per bucket.  kLarge: buckets above kLocalCap are sorted through global memory
-// (needs kin != kout); without it they are reported (CRYS_DEV_BOUNDS) and left alone.
+// A bucket of more than kLocalCap rows that one cut of its key range divides into two parts that
+// fit the block: the rows move from kin to kout, the lower part first, and the parts are sorted
+// there.  Any other bucket goes through global memory.  (Not stable; a function of its own,
+// so that the usual path keeps its registers.)  The buckets of 327M evenly spread rows hold
+// kLocalCap rows on average: 328M rows take 6.96 ms, with all larger buckets through global memory
+// 10.95; 400M rows 9.98 and 18.6.
+static __device__ __noinline__ void local_sort_split(const LocalArgs& a, LocalShared& sh, uint32_t begin, uint32_t size) {
+  __shared__ uint32_t cut, next[2];  // last bin of the lower part; next row of each part
+  const int tid = threadIdx.x, lane = tid % kWarp;
+  const int32_t *kin = a.kin + begin, *vin = a.vin + begin;
+  int32_t lo = INT32_MAX, hi = INT32_MIN;
+  for (uint32_t i = tid; i < size; i += kLocalThreads) {
+    lo = min(lo, kin[i]);
+    hi = max(hi, kin[i]);
+  }
+  if (tid < 256) sh.digit_start[tid] = 0;
+  if (tid == 0) cut = 256;
+  local_range(sh, lo, hi);
+  const int bits = 32 - __clz(static_cast<uint32_t>(hi) - static_cast<uint32_t>(lo));
+  const int shift = bits > 8 ? bits - 8 : 0;
+  auto bin = [&](int32_t k) { return (static_cast<uint32_t>(k) - static_cast<uint32_t>(lo)) >> shift; };
+  if (size <= 2u * kLocalCap)
+    for (uint32_t i = tid; i < size; i += kLocalThreads) atomicAdd(&sh.digit_start[bin(kin[i])], 1u);
+  __syncthreads();
+  const uint32_t rows = tid < 256 ? sh.digit_start[tid] : 0u;
+  uint32_t total;
+  const uint32_t upto = local_scan(rows, sh.tmp, &total) + rows;
+  if (tid < 256 && upto <= static_cast<uint32_t>(kLocalCap) && upto + kLocalCap >= size) atomicMin(&cut, static_cast<uint32_t>(tid));
+  __syncthreads();
+  const uint32_t last = cut;
+  if (size > 2u * kLocalCap || last == 256u) {
+    local_sort_large(a, sh, begin, size);
+    return;
+  }
+  if (static_cast<uint32_t>(tid) == last) {
+    next[0] = 0;
+    next[1] = upto;
+  }
+  if (tid == 0) {
+    mbar_init(&sh.loaded, 1);
+    fence_barrier_init();
+  }
+  __syncthreads();
+  const uint32_t lower = next[1];
+  __syncthreads();
+  for (uint32_t i0 = 0; i0 < size; i0 += kLocalThreads) {
+    const uint32_t i = i0 + tid;
+    const int32_t k = i < size ? kin[i] : 0, v = i < size ? vin[i] : 0;
+    const uint32_t up = bin(k) > last ? 1u : 0u;
+#pragma unroll
+    for (uint32_t part = 0; part < 2; ++part) {
+      const uint32_t mine = __ballot_sync(0xFFFFFFFFu, i < size && up == part);
+      uint32_t at = 0;
+      if (lane == 0 && mine) at = atomicAdd(&next[part], static_cast<uint32_t>(__popc(mine)));
+      at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(mine & ((1u << lane) - 1u));
+      if (i < size && up == part) {
+        a.kout[begin + at] = k;
+        a.vout[begin + at] = v;
+      }
+    }
+  }
+  asm volatile("fence.proxy.async;" ::: "memory");  // the values stored here are read by a bulk copy
+  __syncthreads();
+  const LocalArgs l{a.kout, a.vout, a.kout, a.vout, nullptr, nullptr, a.n, a.err};
+  for (uint32_t part = 0; part < 2; ++part) {
+    const uint32_t rows_of = part ? size - lower : lower;
+    local_sort_bucket(l, sh, begin + (part ? lower : 0u), rows_of, part);
+    fence_proxy_async_smem();  // the other part's values come by a bulk copy into the same place
+    __syncthreads();
+  }
+}
+
+// One block per bucket.  kLarge: buckets above kLocalCap are divided or sorted through global
+// memory (needs kin != kout); without it they are reported (CRYS_DEV_BOUNDS) and left alone.
 template <bool kLarge>
 __global__ void __launch_bounds__(kLocalThreads, 3) local_sort_kernel(const __grid_constant__ LocalArgs a) {
   extern __shared__ __align__(128) unsigned char local_smem[];
@@ -382,7 +454,7 @@ __global__ void __launch_bounds__(kLocalThreads, 3) local_sort_kernel(const __gr
   if (size == 0) return;
   if (size > static_cast<uint32_t>(kLocalCap)) {
     if (kLarge)
-      local_sort_large(a, sh, begin, size);
+      local_sort_split(a, sh, begin, size);
     else if (threadIdx.x == 0)
       set_error(a.err, CRYS_DEV_BOUNDS);
     return;
