@@ -429,6 +429,12 @@ __device__ __forceinline__ uint32_t eval_tile_vectors(const DevQuery& q, const C
   constexpr int VEC = ITEMS / 4;
   constexpr int KP = TileVectors<ITEMS>::KP;
   constexpr int KJ = TileVectors<ITEMS>::KJ;
+  // A tile's code should stay in the instruction cache, so the joins past the second are not
+  // unrolled.  With hashed tables the smaller tiles are an exception: they are for a few tiles
+  // per SM, where the longer code and its 80 registers are faster (four joins, 311,296 rows:
+  // 10.6 us against 11.6 us in 64 registers with spills).
+  constexpr bool kUnroll = !DIRECT && THREADS * ITEMS <= 2048 && ITEMS == 8;
+  constexpr int kPredUnroll = kUnroll ? 4 : 1;
   const int tid = static_cast<int>(threadIdx.x);
   const auto& pv = tv.pv;
   const auto& kv = tv.kv;
@@ -457,7 +463,7 @@ __device__ __forceinline__ uint32_t eval_tile_vectors(const DevQuery& q, const C
   auto join = [&](const DevJoin& J, const int32_t (&key)[ITEMS]) {
     int32_t value[ITEMS];
     alive &= probe_items<ITEMS, DIRECT>(J.slots, J.hash, key, alive, value, pol_table);
-#pragma unroll 1
+#pragma unroll kPredUnroll
     for (int f = 0; f < J.n_fp; ++f) {
       const uint32_t sh = J.fp_shift[f], mk = J.fp_mask[f], span = J.fp_span[f];
       const int32_t lo = J.fp_lo[f];
@@ -489,12 +495,21 @@ __device__ __forceinline__ uint32_t eval_tile_vectors(const DevQuery& q, const C
     for (int j = 0; j < VEC; ++j) unpack4(kv[jn][j], key + 4 * j);
     join(q.joins[jn], key);
   }
-#pragma unroll 1
-  for (int jn = KJ; jn < q.n_joins; ++jn) {  // not unrolled: the code of a tile should stay in the instruction cache
+  auto late_join = [&](int jn) {
     int32_t key[ITEMS];
 #pragma unroll
     for (int j = 0; j < VEC; ++j) unpack4(cols.load4(q.joins[jn].fk_col, (j * THREADS + tid) * 4), key + 4 * j);
     join(q.joins[jn], key);
+  };
+  if constexpr (kUnroll) {
+#pragma unroll
+    for (int jn = KJ; jn < CRYS_MAX_JOINS; ++jn) {
+      if (jn >= q.n_joins) break;
+      late_join(jn);
+    }
+  } else {
+#pragma unroll 1
+    for (int jn = KJ; jn < q.n_joins; ++jn) late_join(jn);
   }
 #pragma unroll
   for (int j = 0; j < VEC; ++j) {
@@ -1852,11 +1867,17 @@ bool of_fixed_shape(const DevQuery& q) {
          (q.agg_op == CRYS_AGG_A_MUL_B || q.agg_op == CRYS_AGG_A);
 }
 
-// Without a shape set, any plan takes the smaller tiles while these are at most one per SM: half
-// as many larger ones leave the other SMs idle (three joins on direct tables, 100,003 rows: 6.4
-// us with 256 x 8, 7.9 with 512 x 8; 311,296 rows 6.5 and 7.9; 400,003 rows, on more than one
-// tile for some SMs, 8.2 and 8.0).
-bool one_small_tile_per_sm(int64_t rows) { return rows <= static_cast<int64_t>(sm_count()) * 256 * 8; }
+// Without a shape set, any plan takes the smaller tiles where the SM with the most of them then
+// has at most three quarters of the rows that it has in larger ones.  That is up to one per SM
+// (three joins on direct tables, 100,003 rows: 6.4 us with 256 x 8, 7.9 with 512 x 8; 311,296 rows
+// 6.5 and 7.9; 400,003 rows, two per SM or one, 8.2 and 8.0), and where the larger ones just
+// exceed one per SM (800,003 rows 10.4 and 11.8; 1,000,003 rows 12.1 and 11.9).
+bool smaller_tiles_balance(int64_t rows) {
+  constexpr int64_t kLarge = 512 * 8, kSmall = 256 * 8;
+  const int64_t large = ((rows + kLarge - 1) / kLarge + sm_count() - 1) / sm_count() * kLarge;
+  const int64_t small = ((rows + kSmall - 1) / kSmall + sm_count() - 1) / sm_count() * kSmall;
+  return 4 * small <= 3 * large;
+}
 
 // Rows up to which, without a shape set, plans of the Q1 family take the smaller tiles: the
 // last tiles of so few rows leave much of the chip idle (12,000,001 rows 31.4 us with 256 x 8,
@@ -2463,9 +2484,10 @@ int crys_run_plan(const crys_table* fact, const crys_plan* plan, crys_stream str
     case 2: return launch_plan<kTiles[kOp][2].threads, kTiles[kOp][2].items>(a, s);
     case 3: return launch_plan<kTiles[kOp][3].threads, kTiles[kOp][3].items>(a, s);
     default:
-      static_assert(kTiles[kOp][1].threads == 256 && kTiles[kOp][1].items == 8, "the default shape's smaller tiles");
+      static_assert(kTiles[kOp][0].threads == 512 && kTiles[kOp][0].items == 8 && kTiles[kOp][1].threads == 256 &&
+                        kTiles[kOp][1].items == 8, "the larger and the smaller tiles");
       if (set_tile_variant(kOp) < 0 &&
-          (one_small_tile_per_sm(fact->n_rows) || (fact->n_rows <= kSmallTileRows && of_fixed_shape(a.q))))
+          (smaller_tiles_balance(fact->n_rows) || (fact->n_rows <= kSmallTileRows && of_fixed_shape(a.q))))
         return launch_plan<kTiles[kOp][1].threads, kTiles[kOp][1].items>(a, s);
       return launch_plan<kTiles[kOp][0].threads, kTiles[kOp][0].items>(a, s);
   }

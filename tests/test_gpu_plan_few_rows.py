@@ -1,6 +1,6 @@
-"""Queries over tables of few rows, at the edges of the default shape's rule: up to 2048 rows per
-SM in tiles of 2048 rows, above in tiles of 4096; one to three joins on direct and hashed
-tables, grouped, against the oracle."""
+"""Queries over tables of few rows, at the edges of the library's own choice of tiles: up to 2048
+rows per SM in tiles of 2048 rows, up to 4096 in tiles of 4096, up to 6144 in the smaller
+ones again; one to three joins on direct and hashed tables, grouped."""
 import numpy as np
 import pytest
 
@@ -24,10 +24,14 @@ def crys():
 
 @pytest.mark.parametrize("direct", [True, False])
 @pytest.mark.parametrize("joins", [1, 2, 3])
-@pytest.mark.parametrize("rows", [1, 2049, "line-1", "line", "line+1", "line+4097"])
+@pytest.mark.parametrize("rows", [1, 2049, "line-1", "line", "line+1", "line+4097", "2line", "2line+1", "3line", "3line+1"])
 def test_plans_of_few_rows(crys, rows, joins, direct):
     line = torch.cuda.get_device_properties(0).multi_processor_count * 2048
-    n = rows if isinstance(rows, int) else line + int(rows[4:] or 0)
+    if isinstance(rows, int):
+        n = rows
+    else:
+        times, _, more = rows.partition("line")
+        n = int(times or 1) * line + int(more or 0)
     g = torch.Generator(device="cuda")
     g.manual_seed(n + joins)
 
