@@ -770,8 +770,9 @@ extern "C" int crys_sort_msb(const int32_t* keys_in, const int32_t* vals_in, int
   if (bits == 0)  // one block sorts everything
     return launch_local_sort<false>(LocalArgs{keys_in, vals_in, keys_out, vals_out, nullptr, nullptr, rows, err}, 1, s);
   // (its counts lie in the output's keys, read in 16-byte groups)
-  if (aligned16(keys_out) && small_sort_fits(n))
-    return launch_small_sort(keys_in, vals_in, tk, tv, keys_out, vals_out, n, range, s);
+  if (aligned16(keys_out) && small_sort_fits(n) &&
+      launch_small_sort(keys_in, vals_in, tk, tv, keys_out, vals_out, n, range, s) == CRYS_OK)
+    return CRYS_OK;  // (refused on a stream that owns few SMs: by a pass)
   if (launch_key_range(keys_in, n, bits, range, nullptr, s) != CRYS_OK) return CRYS_ECUDA;
   // level A: the whole array by the leading 8 bits
   seg_init_kernel<<<1, 1, 0, s>>>(rows, kPartTile, A.seg_begin, A.seg_size, A.tile_start);

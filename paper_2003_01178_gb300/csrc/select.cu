@@ -645,8 +645,10 @@ extern "C" int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, 
     select_small_kernel<<<kSmallBlocks, kSmallThreads, smem, s>>>(x, static_cast<int>(n), lo,
                                                               static_cast<uint32_t>(hi) - static_cast<uint32_t>(lo), out,
                                                               reinterpret_cast<long long*>(d_count), err);
-    note_launch();
-    return check_launch();
+    if (check_launch() == CRYS_OK) {
+      note_launch();
+      return CRYS_OK;
+    }  // a cluster this large was refused (a stream that owns few SMs): by tiles
   }
   if (cudaMemsetAsync(d_count, 0, sizeof(int64_t), s) != cudaSuccess) return CRYS_ECUDA;
   if (n == 0) return CRYS_OK;

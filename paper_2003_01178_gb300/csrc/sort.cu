@@ -701,9 +701,10 @@ extern "C" int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t
     return launch_local_sort<false>(
         LocalArgs{keys_in, vals_in, keys_out, vals_out, nullptr, nullptr, static_cast<uint32_t>(n), err}, 1, s);
   }
-  if (!stalled && any_tile && small_sort_fits(n))
-    return launch_small_sort(keys_in, vals_in, reinterpret_cast<int32_t*>(temp + L.tmp_keys),
-                             reinterpret_cast<int32_t*>(temp + L.tmp_vals), keys_out, vals_out, n, temp + L.counters, s);
+  if (!stalled && any_tile && small_sort_fits(n) &&
+      launch_small_sort(keys_in, vals_in, reinterpret_cast<int32_t*>(temp + L.tmp_keys),
+                        reinterpret_cast<int32_t*>(temp + L.tmp_vals), keys_out, vals_out, n, temp + L.counters, s) == CRYS_OK)
+    return CRYS_OK;  // (refused on a stream that owns few SMs: by passes)
   // up to 2^20 rows (one pass by buckets) the smallest tile, so that more SMs have one
   switch (any_tile && n <= (1 << 20) ? kNumVariants[kOp] - 1 : tile_variant(kOp)) {
     case 1: return run_sort<kTiles[kOp][1].threads, kTiles[kOp][1].items>(keys_in, vals_in, keys_out, vals_out, n, temp, L, stall_base, stall_ns, s);
