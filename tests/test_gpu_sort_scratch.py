@@ -63,3 +63,17 @@ def test_one_scratch(crys, n, variant):
         rk, order = torch.sort(keys, stable=True)
         assert torch.equal(ko, rk) and torch.equal(vo, order.to(torch.int32)), kind
     crys.crys_set_tile(crys.OP_SORT, 0)
+
+
+def test_more_rows_than_the_buckets_take(crys):
+    # above 2^28 rows every stable sort goes by digits
+    n = (1 << 28) + 77
+    keys = torch.randint(I32_MIN, I32_MAX, (n,), dtype=torch.int32, device="cuda")
+    vals = torch.arange(n, dtype=torch.int32, device="cuda")
+    ko, vo = crys.sort(keys, vals)
+    assert bool((ko[1:] >= ko[:-1]).all()) and torch.equal(keys[vo.long()], ko)
+    equal = ko[1:] == ko[:-1]
+    assert bool((vo[1:][equal] > vo[:-1][equal]).all())
+    seen = torch.zeros(n, dtype=torch.bool, device="cuda")
+    seen[vo.long()] = True
+    assert bool(seen.all())
