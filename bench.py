@@ -637,12 +637,26 @@ def op_q1(args, dev, stream, sizes):
                                            "speedup_over_dense_query": round(ms / sms, 3)}
         del t, f, d, ht, table, plan, sel
     del flush_buf
-    return {"kernel": "plan_kernel", "by_rows": out, "bytes": "16 B per fact row: 4 columns (Section 3.1 bound)",
+    return {"kernel": "plan_fixed_kernel", "by_rows": out, "bytes": "16 B per fact row: 4 columns (Section 3.1 bound)",
             "plan": "the 2556-row date dimension in a direct table (perfect hashing of the dense keys) filtered "
                     "on yr == 3, probed by one fused kernel",
             "l2": "flushed before each timed launch (512 MB write)",
             "graph_ms_note": "per-launch device time from CUDA-graph replays of k x {L2 flush, kernel} minus "
                              "k x {L2 flush}: no launch or event overhead"}
+
+
+def sort_traffic(crys, n):
+    """(bytes, what they are, passes) of a stable sort of n random keys, by the way that it takes."""
+    shape_set = crys.crys_tile_is_set(crys.OP_SORT)
+    if n <= 1 << 20 and not shape_set:
+        return 32 * n, "one launch: rows to buckets, buckets sorted, each 8N read + 8N written = 32N", "one launch"
+    by_digits = n > 1 << 28 or n <= 4992 or crys.crys_tile_variants(crys.OP_SORT)[crys.crys_get_tile(crys.OP_SORT)] == (256, 16)
+    if by_digits:
+        return 68 * n, "one 4N key read for all digit histograms + 4 passes x (8N read + 8N written) = 68N", "4 x 8-bit, stable"
+    passes = 1 if n <= 1 << 20 else 2
+    return (20 + 16 * passes) * n, (f"one 4N key read for the bucket counts + {passes} x (8N read + 8N written) + bucket "
+                                    f"sort (8N read + 8N written) = {20 + 16 * passes}N"), \
+        f"{passes} x 8-bit, stable, and a sort inside every bucket"
 
 
 def op_sort(args, dev, stream, n=1 << 28):
@@ -659,11 +673,10 @@ def op_sort(args, dev, stream, n=1 << 28):
     tile = autotune(crys.OP_SORT, lambda: crys.crys_sort(keys, vals, ko, vo, n, temp, tb), args)
     ms = statistics.median(time_launches(lambda: crys.crys_sort(keys, vals, ko, vo, n, temp, tb),
                                          args.steps, args.warmup, stream))
+    nbytes, what, passes = sort_traffic(crys, n)
     res = {"kernel": "sort_pass_kernel", "rows": n, "lsd_stable": {
-        "ms": round(ms, 4), "Mkeys/s": round(n / (ms / 1e3) / 1e6, 1), "GB/s": round(gbs(52 * n, ms), 1),
-        "frac": frac(52 * n, ms), "tile": tile,
-        "bytes": "one 4N key read for the bucket counts + 2 passes x (8N read + 8N written) + bucket sort "
-                 "(8N read + 8N written) = 52N"},
+        "ms": round(ms, 4), "Mkeys/s": round(n / (ms / 1e3) / 1e6, 1), "GB/s": round(gbs(nbytes, ms), 1),
+        "frac": frac(nbytes, ms), "tile": tile, "alg_bytes": nbytes, "bytes": what, "passes": passes},
         "paper": "V100: 27.08 ms for 2^28 key+value pairs, unstable MSB sort (Section 4.4)"}
     del temp
     # the paper's own GPU sort: most-significant-digit first, unstable
@@ -822,17 +835,15 @@ def run_operator(args, rank, world, local):
         elif args.workload == "sort":
             r = op_sort(args, dev, stream, args.rows or (1 << 28))
             s = r["lsd_stable"]
-            line = op_line(args, world, "sort", s["Mkeys/s"], "Mkeys/s", "sort_pass_kernel", 52 * r["rows"], s["ms"],
-                           {"rows": r["rows"], "l2": "inputs larger than L2", "passes": "4 x 8-bit, stable"},
+            line = op_line(args, world, "sort", s["Mkeys/s"], "Mkeys/s", "sort_pass_kernel", s["alg_bytes"], s["ms"],
+                           {"rows": r["rows"], "l2": "inputs larger than L2", "passes": s["passes"]},
                            {"sort": r})
         elif args.workload == "q1":
             sizes = [args.rows] if args.rows else [1 << 22, 1 << 28]
             r = op_q1(args, dev, stream, sizes)
             n = sizes[0]
             q = r["by_rows"][str(n)]
-            # the library runs the kernel compiled for this plan's shape when each block takes
-            # at most 8 tiles (every tile shape at 2^22 rows), the generic one otherwise
-            kernel = "plan_fixed_kernel" if n <= (1 << 22) else "plan_kernel"
+            kernel = "plan_fixed_kernel"       # the one compiled for this plan's shape, at every size
             per_call = q["graph_ms"] if q.get("graph_ms") else q["ms"]
             line = op_line(args, world, "q1", q["GB/s"], "GB/s", kernel, 16 * n, per_call,
                            {"rows": n, "dtype": "int64", "l2": "flushed between timed launches (512 MB write)",

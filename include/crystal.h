@@ -49,7 +49,7 @@ typedef struct CUstream_st* crys_stream; /* the same type as cudaStream_t */
 #define CRYS_ECUDA (-5)    /* a CUDA runtime call failed (launch or memset) */
 
 /* Bits of the per-device error word (crys_device_errors). */
-#define CRYS_DEV_TIMEOUT 0x1    /* a bounded spin-wait (mbarrier, look-back) gave up */
+#define CRYS_DEV_TIMEOUT 0x1    /* a bounded spin-wait (mbarrier, other blocks) gave up */
 #define CRYS_DEV_TABLE_FULL 0x2 /* an insert probed the whole table without a free slot */
 #define CRYS_DEV_BAD_KEY 0x4    /* key -1 (0xFFFFFFFF, the empty-slot marker) on build */
 #define CRYS_DEV_DUP_KEY 0x8    /* a build key was inserted twice */
@@ -69,7 +69,7 @@ int64_t crys_launch_count(void);
 /* Test hook for the bounded waits (failure detection; the paper has no counterpart).
  * The NEXT call of `op` in this process - an order-preserving crys_select (also through
  * crys_select_static) or a crys_sort - hands out tile ids starting at `first_tile`
- * instead of 0 and bounds its look-back waits by `wait_limit_ns` (1 us .. 2 s) instead
+ * instead of 0 and bounds its waits between tiles by `wait_limit_ns` (1 us .. 2 s) instead
  * of 2 s.  With first_tile > 0 the tiles before it never publish their counts, so the
  * tile after them waits for a flag that nothing sets: the call's blocks give up once
  * the bound has passed, CRYS_DEV_TIMEOUT is set in the device error word and the call's
@@ -103,7 +103,7 @@ int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, int32_t* ou
  * query executors and plugins that run inside a host process owning a fixed,
  * pre-reserved device memory pool, or real-time pipelines that forbid allocation after
  * start-up).  Same result as crys_select(..., order_preserving = 1, ...), but the
- * look-back scratch lives in a file-scope static device array of the library
+ * tiles' status words live in a file-scope static device array of the library
  * (CRYS_SELECT_STATIC_SCRATCH_BYTES bytes, held by every device that loads the
  * library until the process exits).  The caller still passes x, out and d_count.
  *   n > CRYS_SELECT_STATIC_MAX_ROWS returns CRYS_EINVAL (nothing enqueued).
@@ -200,9 +200,9 @@ int crys_probe_aggregate(const int32_t* fk, const int32_t* payload, int64_t n,
  * then sorted inside one thread block; other keys take a least-significant-digit sort, a
  * pass per 8-bit digit that varies.  The choice is made on the device.  Each pass ranks a
  * tile stably inside the thread block and finds the tile's output offsets with a chained
- * scan over the tiles.  More than 2^28 rows always take a pass per digit.  Up to 4992 rows
- * are sorted by one block and up to 2^20 rows by one cooperative launch (while no tile shape
- * is set).  n <= 2^30 - 1.
+ * scan over the tiles.  More than 2^28 rows, or the tile shape 256 x 16, always take a pass
+ * per digit.  Up to 4992 rows are sorted by one block and up to 2^20 rows by one cooperative
+ * launch (while no tile shape is set).  n <= 2^30 - 1.
  * keys_out/vals_out must not overlap the inputs; the inputs are not modified. */
 int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out,
               int32_t* vals_out, int64_t n, void* d_temp, size_t* temp_bytes, crys_stream s);
@@ -212,8 +212,9 @@ int crys_sort(const int32_t* keys_in, const int32_t* vals_in, int32_t* keys_out,
  * keys_out is 16-byte aligned; one partition pass if not), above that two partition passes
  * of at most 8 bits, each a histogram, a scan and a scatter whose tiles rank their keys with
  * shared-memory atomics and reserve each digit's run with one global atomic; then every
- * bucket is sorted inside one thread block by its remaining bits and stored.  The passes' bits are those of a key's place between the smallest and the largest
- * key of a sample, so narrow key ranges fill the buckets like wide ones.
+ * bucket is sorted inside one thread block by its remaining bits and stored.  The passes' bits
+ * are those of a key's place between the smallest and the largest key of a sample, so narrow
+ * key ranges fill the buckets like wide ones.
  * Keys come out in ascending signed order; rows with EQUAL keys may come out in any order
  * (unstable), so (key, value) pairs are a permutation of the input pairs.  A bucket of
  * more than 4992 rows (heavily repeated or clustered keys, or more than about 315M rows) is

@@ -182,7 +182,7 @@ def crys_launch_count() -> int:
 
 def crys_debug_stall(op: int, first_tile: int, wait_limit_ns: int) -> None:
     """Test hook: the next order-preserving select or sort starts its tile ids at
-    first_tile (earlier tiles never publish) and bounds its look-back waits."""
+    first_tile (earlier tiles never publish) and bounds its waits between tiles."""
     _check(lib().crys_debug_stall(op, first_tile, wait_limit_ns), "crys_debug_stall")
 
 

@@ -24,7 +24,7 @@ int tile_variant(int op);
 int set_tile_variant(int op);
 
 // The stall requested by crys_debug_stall for the next call of `op`, consumed by this
-// call: tile ids start at *first_tile and look-back waits give up after *wait_ns.
+// call: tile ids start at *first_tile and waits between tiles give up after *wait_ns.
 // Without a request: 0 and the default bound.  Returns whether a request was taken.
 bool take_stall(int op, uint32_t* first_tile, uint64_t* wait_ns);
 

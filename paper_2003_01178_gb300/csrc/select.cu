@@ -46,7 +46,7 @@ struct SelectArgs {
   unsigned int* block_counter; // mode 1: blocks that have started (the first one scans)
   unsigned int* abort_word;   // mode 1: set by the first block of this call that gives up
   uint32_t tile_base;         // mode 1: first tile id handed out (0 unless a test stalls)
-  uint64_t wait_ns;           // mode 1: bound of a look-back wait
+  uint64_t wait_ns;           // mode 1: bound of a wait for a count or a position
   int32_t* err;
   int32_t stages;
 };
@@ -695,7 +695,7 @@ extern "C" int crys_select(const int32_t* x, int64_t n, int32_t lo, int32_t hi, 
 }
 
 // ---------------------------------------------------------------------------
-// Allocation-free order-preserving selection: the look-back scratch is a static device
+// Allocation-free order-preserving selection: the tiles' status words are a static device
 // array of this file instead of caller-supplied memory.
 
 namespace crys {
@@ -738,6 +738,6 @@ extern "C" int crys_select_static(const int32_t* x, int64_t n, int32_t lo, int32
   void* scratch = static_scratch();
   if (!scratch) return CRYS_ECUDA;
   size_t have = CRYS_SELECT_STATIC_SCRATCH_BYTES;
-  // crys_select clears the `need` bytes it uses on `stream` before its kernel runs.
+  // crys_select clears the words it uses (none for a column of one cluster) on `stream` first.
   return crys_select(x, n, lo, hi, out, d_count, 1, scratch, &have, stream);
 }

@@ -2,8 +2,8 @@
 // stable).  The steps of the larger sort would be a dozen launches and clearings here, and the
 // host needs 3 to 4 us for each; the work itself takes less.
 //
-// A cooperative launch of at most 304 blocks, each holding up to 4992 rows, with a grid
-// barrier between the steps:
+// A cooperative launch of a block per SM (fewer for few rows, up to 211 where the blocks would
+// hold too many), each holding up to 4992 rows, with a grid barrier between the steps:
 //  1. smallest and largest key;
 //  2. every block ranks its rows stably by the bucket of their key (up to 256 buckets over the
 //     key range) and publishes its bucket counts;
@@ -15,8 +15,8 @@
 // key - smallest instead, from the low one to the high one (each block takes its rows of the
 // previous digit's result again).
 //
-// 100,003 random pairs: 60 us per call with the larger sort's steps, 28 us here; 2^20 pairs: 84
-// and 48 us.  What bounds it is latency: three grid barriers of about 2 us each and a few
+// 100,003 random pairs: 60 us per call with the larger sort's steps, 22 us here; 2^20 pairs: 84
+// and 46 us.  What bounds it is latency: three grid barriers of about 2 us each and a few
 // dependent trips to L2 between them, at one block per SM.
 #include "common.cuh"
 #include "localsort.cuh"

@@ -9,9 +9,9 @@
 //    gives the passes' bucket starts and shows whether any bucket is too large for a block.
 //  * digits: when one is (heavily repeated or clustered keys), when a sample of the keys differs
 //    in at most three bytes or shows more than eight rows per key value (keyrange.cuh), or
-//    when there are too many rows, the
-//    least-significant-digit sort: 8-bit digits, a stable pass per digit from the low one to
-//    the high one.  Digits that have one value in all keys are skipped.
+//    when there are too many rows, the least-significant-digit sort: 8-bit digits, a stable
+//    pass per digit from the low one to the high one.  Digits that have one value in all
+//    keys are skipped.
 //
 // A pass is ONE kernel: a thread block takes the next tile id from an atomic counter, ranks
 // its keys stably inside the block (per-warp multisplit: keys are processed warp-striped,
@@ -285,9 +285,9 @@ struct PassArgs {
   int pass;
   SortHead* head;
   const unsigned int* digit_base;  // 256 bucket starts of this pass
-  uint32_t* status;                // per tile x digit look-back words
+  uint32_t* status;                // per tile x digit: the tile's count, then its position
   uint32_t tile_base;              // first tile id handed out (0 unless a test stalls)
-  uint64_t wait_ns;                // bound of a look-back wait
+  uint64_t wait_ns;                // bound of a wait for a count or a position
   int32_t* err;
 };
 
